@@ -305,6 +305,7 @@ struct mppi_ctx {
   int n = 3;
   int Jcap = 0;
   int smem = 0;
+  int nc = 0;  // far-field cells of a tile
   CtrlDesc D;
   StepFn fn = nullptr;
   double* d_U = nullptr;
@@ -389,7 +390,7 @@ void free_ctx(mppi_ctx* c) {
 // least twice when K allows, then shrunk until the tile's shared memory
 // (whole-horizon poses and controls, obstacles) fits.
 int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tiling* out,
-                  int* smem_out, bool batched = false) {
+                  int* smem_out, int* nc_out, bool batched = false) {
   const int sms = num_sms();
   const int n = state_dim(p->model);
   mppi_tiling t = {0, 0, 0, 0};
@@ -415,8 +416,15 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
     const int GT = group_size(nTiles);
     const int nGroups = (nTiles + GT - 1) / GT;
     const int nscl = GT > nGroups ? GT : nGroups;
-    SmemLayout L =
-        smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, batched);
+    // with far-field cells where they fit, else without them
+    const int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads);
+    SmemLayout L = smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, nc,
+                               batched);
+    *nc_out = nc;
+    if (L.total > limit && nc > 0) {
+      L = smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, 0, batched);
+      *nc_out = 0;
+    }
     if (L.total <= limit) {
       *smem_out = L.total;
       break;
@@ -445,14 +453,13 @@ void fill_desc(mppi_ctx* c) {
   D.n = c->n;
   D.S = c->tl.samples_per_cta;
   D.NPOS = c->tl.positions_per_thread;
+  D.nc = c->nc;
   D.nTiles = (p->K + D.S - 1) / D.S;
   D.GT = group_size(D.nTiles);
   D.nGroups = (D.nTiles + D.GT - 1) / D.GT;
   D.nscl = D.GT > D.nGroups ? D.GT : D.nGroups;
   D.dt = (float)p->dt;
   D.h_eps = (float)p->h_eps;
-  D.gamma_bas_f = (float)p->gamma_bas;
-  D.R_B = (float)p->R_B;
   D.C_coll = (float)p->C_coll;
   D.ln_mu = (float)p->ln_mu;
   D.ln_sigma = (float)p->ln_sigma;
@@ -469,19 +476,18 @@ void fill_desc(mppi_ctx* c) {
   }
   for (int i = 0; i < 2 * kMaxShape; ++i)
     D.shape[i] = i < 2 * p->n_shape ? (float)p->shape[i] : 0.0f;
+  D.r_body = 0.0f;
+  for (int i = 0; i < p->n_shape; ++i)
+    D.r_body = std::max(D.r_body, 1.000001f * std::hypot(D.shape[2 * i], D.shape[2 * i + 1]));
   D.g = (float)p->gravity;
   D.inv_mass = (p->model == MPPI_QUAD2D || p->model == MPPI_QUAD5) ? (float)(1.0 / p->mass) : 0.0f;
   D.k_turn = p->model == MPPI_QUAD2D      ? (float)(p->arm / p->inertia)
              : p->model == MPPI_ACKERMANN ? (float)(1.0 / p->wheelbase)
                                           : 0.0f;
-  D.lambda = p->lambda;
-  D.inv_lambda = 1.0 / p->lambda;
   D.inv_lambda_f = (float)(1.0 / p->lambda);
   D.mu_coarse = p->mu_coarse;
-  D.gamma_ctrl = p->gamma_ctrl;
   D.gamma_bas = p->gamma_bas;
   D.R_B_d = p->R_B;
-  for (int i = 0; i < 4; ++i) D.sigma[i] = p->sigma[i];
   {
     // chol(Sigma) and gamma Sigma^-1 (PSD checked by validate; inverse only
     // needed, and only defined, when gamma_ctrl != 0)
@@ -544,7 +550,7 @@ int mppi_create_tiled(const mppi_params* p, const double* u_init, const mppi_til
   if (!c) return fail(MPPI_ENOMEM, "host allocation failed");
   c->p = *p;
   c->n = state_dim(p->model);
-  rc = choose_tiling(p, tiling, 0, &c->tl, &c->smem);
+  rc = choose_tiling(p, tiling, 0, &c->tl, &c->smem, &c->nc);
   if (rc) {
     delete c;
     return rc;
@@ -651,8 +657,8 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
     if (int rc = check_obstacle(cxcyr + 3 * j, j)) return rc;
   }
   mppi_tiling t;
-  int smem = 0;
-  int rc = choose_tiling(&c->p, &c->tl, J, &t, &smem);
+  int smem = 0, nc = 0;
+  int rc = choose_tiling(&c->p, &c->tl, J, &t, &smem, &nc);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->last));
   const size_t bytes = (size_t)align_up(24 * (J > 0 ? J : 1), 16);
@@ -678,8 +684,10 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   if (rc) return rc;
   c->tl = t;
   c->smem = smem;
+  c->nc = nc;
   c->fn = fn;
   c->D.J = J;
+  c->D.nc = nc;
   c->D.obst = c->d_obst;
   return MPPI_OK;
 }
@@ -1071,7 +1079,7 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   mppi_ctx c;  // on the stack: only its descriptor logic is used
   c.p = *p;
   c.n = state_dim(p->model);
-  rc = choose_tiling(p, nullptr, J, &c.tl, &c.smem);
+  rc = choose_tiling(p, nullptr, J, &c.tl, &c.smem, &c.nc);
   if (rc) return rc;
   const int T = p->T, K = p->K;
   const int nTiles = (K + c.tl.samples_per_cta - 1) / c.tl.samples_per_cta;
@@ -1282,7 +1290,7 @@ struct BatchSlot {
   bool used = false;
   mppi_params p;
   mppi_tiling tl;
-  int n = 3, J = 0, Jcap = 0, smem = 0;
+  int n = 3, J = 0, Jcap = 0, smem = 0, nc = 0;
   size_t off = 0, bytes = 0;   // pool range
   size_t obst_off = 0;         // pool offset of the obstacle area
   CtrlDesc D;
@@ -1492,6 +1500,7 @@ int batch_write_desc(mppi_batch* b, int slot) {
   c.p = s.p;
   c.n = s.n;
   c.tl = s.tl;
+  c.nc = s.nc;
   slot_layout(b, s, &c);
   fill_desc(&c);
   c.D.J = s.J;
@@ -1566,7 +1575,7 @@ int mppi_batch_add(mppi_batch* b, const mppi_params* p, const double* u_init,
   if (req.samples_per_cta <= 0) req.samples_per_cta = 32;
   if (req.samples_per_cta > p->K) req.samples_per_cta = p->K;
   int smem = 0;
-  rc = choose_tiling(p, &req, J, &s.tl, &smem, true);
+  rc = choose_tiling(p, &req, J, &s.tl, &smem, &s.nc, true);
   if (rc) return rc;
   if (smem > batch_max_smem(b)) return fail(MPPI_EINVAL, "controller too large for the batch kernel");
   s.J = J;
@@ -1625,8 +1634,8 @@ int mppi_batch_set_obstacles(mppi_batch* b, int32_t slot, const double* cxcyr, i
   }
   BatchSlot& s = b->slots[slot];
   mppi_tiling t;
-  int smem = 0;
-  int rc = choose_tiling(&s.p, &s.tl, J, &t, &smem, true);
+  int smem = 0, nc = 0;
+  int rc = choose_tiling(&s.p, &s.tl, J, &t, &smem, &nc, true);
   if (rc) return rc;
   if (smem > batch_max_smem(b)) return fail(MPPI_EINVAL, "obstacle set too large");
   if (b->lane.last) CK(cudaStreamSynchronize(b->lane.last));
@@ -1644,6 +1653,7 @@ int mppi_batch_set_obstacles(mppi_batch* b, int32_t slot, const double* cxcyr, i
   }
   s.J = J;
   s.smem = smem;
+  s.nc = nc;
   rc = batch_write_desc(b, slot);
   if (rc) return rc;
   if (J > 0) {

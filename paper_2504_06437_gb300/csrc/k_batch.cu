@@ -5,12 +5,11 @@
 
 namespace dbm {
 
-__global__ void __launch_bounds__(kBatchThreads) batch_kernel(const CtrlDesc* __restrict__ descs,
+__global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const CtrlDesc* __restrict__ descs,
                                                               unsigned char* stage,
                                                               double* __restrict__ u0_out) {
-  extern __shared__ __align__(16) char smem[];
-  __shared__ TileScratch ts;
-  __shared__ CtrlDesc Ds;
+  TileScratch& ts = tile_scratch();
+  CtrlDesc& Ds = tile_desc();
   __shared__ int s_item;
   BatchHdr* hdr = reinterpret_cast<BatchHdr*>(stage);
   const StepEntry* steps = reinterpret_cast<const StepEntry*>(stage + sizeof(BatchHdr));
@@ -37,10 +36,10 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const CtrlDesc* __
     double* uo = u0_out + 8 * w.ctrl;  // u0 and the predicted next state
     // the batched form of the tile: see run_tile
     switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-      case 0: run_tile<0, 8, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 1: run_tile<0, 14, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 2: run_tile<1, 8, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      default: run_tile<1, 14, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
+      case 0: run_tile<0, 8>(w.tile, x0, xref, phase, uo); break;
+      case 1: run_tile<0, 14>(w.tile, x0, xref, phase, uo); break;
+      case 2: run_tile<1, 8>(w.tile, x0, xref, phase, uo); break;
+      default: run_tile<1, 14>(w.tile, x0, xref, phase, uo); break;
     }
     __syncthreads();  // Ds and s_item are reused by the next item
   }
@@ -48,7 +47,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const CtrlDesc* __
 
 // Resident serving kernel over the same tile instantiations (see
 // serve_body in kernels.cuh).
-__global__ void __launch_bounds__(kBatchThreads) serve_kernel(const CtrlDesc* __restrict__ descs,
+__global__ void __launch_bounds__(kBatchThreads, 2) serve_kernel(const CtrlDesc* __restrict__ descs,
                                                               ServeRing R) {
   serve_body<false>(descs, R);
 }

@@ -13,9 +13,8 @@ namespace dbm {
 // CTA per SM).
 __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel_all(
     const CtrlDesc* __restrict__ descs, unsigned char* stage, double* __restrict__ u0_out) {
-  extern __shared__ __align__(16) char smem[];
-  __shared__ TileScratch ts;
-  __shared__ CtrlDesc Ds;
+  TileScratch& ts = tile_scratch();
+  CtrlDesc& Ds = tile_desc();
   __shared__ int s_item;
   BatchHdr* hdr = reinterpret_cast<BatchHdr*>(stage);
   const StepEntry* steps = reinterpret_cast<const StepEntry*>(stage + sizeof(BatchHdr));
@@ -42,14 +41,14 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel_all(
     double* uo = u0_out + 8 * w.ctrl;  // u0 and the predicted next state
     // the batched form of the tile: see run_tile
     switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-      case 0: run_tile<0, 8, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 1: run_tile<0, 14, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 2: run_tile<1, 8, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 3: run_tile<1, 14, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 4: run_tile<2, 8, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 5: run_tile<2, 14, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      case 6: run_tile<3, 8, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
-      default: run_tile<3, 14, true>(Ds, w.tile, x0, xref, smem, ts, phase, uo); break;
+      case 0: run_tile<0, 8>(w.tile, x0, xref, phase, uo); break;
+      case 1: run_tile<0, 14>(w.tile, x0, xref, phase, uo); break;
+      case 2: run_tile<1, 8>(w.tile, x0, xref, phase, uo); break;
+      case 3: run_tile<1, 14>(w.tile, x0, xref, phase, uo); break;
+      case 4: run_tile<2, 8>(w.tile, x0, xref, phase, uo); break;
+      case 5: run_tile<2, 14>(w.tile, x0, xref, phase, uo); break;
+      case 6: run_tile<3, 8>(w.tile, x0, xref, phase, uo); break;
+      default: run_tile<3, 14>(w.tile, x0, xref, phase, uo); break;
     }
     __syncthreads();  // Ds and s_item are reused by the next item
   }

@@ -209,9 +209,8 @@ __device__ __forceinline__ int npos_code(int npos) { return npos == 14 ? 1 : 0; 
 // the claim's system-scope acquire and a fence, so it is the latest.
 template <bool ALL>
 __device__ __forceinline__ void serve_body(const CtrlDesc* __restrict__ descs, const ServeRing& R) {
-  extern __shared__ __align__(16) char smem[];
-  __shared__ TileScratch ts;
-  __shared__ CtrlDesc Ds;
+  TileScratch& ts = tile_scratch();
+  CtrlDesc& Ds = tile_desc();
   __shared__ int s_cls;
   __shared__ unsigned s_idx;
   __shared__ __align__(16) double s_in[kServeInputMax];
@@ -243,17 +242,17 @@ __device__ __forceinline__ void serve_body(const CtrlDesc* __restrict__ descs, c
     const double* x0 = s_in;
     const double* xref = s_in + xref_off;
     switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-      case 0: run_tile<0, 8, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
-      case 1: run_tile<0, 14, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
-      case 2: run_tile<1, 8, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
-      case 3: run_tile<1, 14, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
+      case 0: run_tile<0, 8>(tile, x0, xref, phase, uo); break;
+      case 1: run_tile<0, 14>(tile, x0, xref, phase, uo); break;
+      case 2: run_tile<1, 8>(tile, x0, xref, phase, uo); break;
+      case 3: run_tile<1, 14>(tile, x0, xref, phase, uo); break;
       default:
         if constexpr (ALL) {
           switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-            case 4: run_tile<2, 8, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
-            case 5: run_tile<2, 14, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
-            case 6: run_tile<3, 8, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
-            default: run_tile<3, 14, true>(Ds, tile, x0, xref, smem, ts, phase, uo); break;
+            case 4: run_tile<2, 8>(tile, x0, xref, phase, uo); break;
+            case 5: run_tile<2, 14>(tile, x0, xref, phase, uo); break;
+            case 6: run_tile<3, 8>(tile, x0, xref, phase, uo); break;
+            default: run_tile<3, 14>(tile, x0, xref, phase, uo); break;
           }
         }
         break;
@@ -272,12 +271,11 @@ __device__ __forceinline__ void serve_body(const CtrlDesc* __restrict__ descs, c
 template <int MODEL, int NPOS, bool SGF = false, bool GRID = false>
 __device__ __forceinline__ void step_body(const CtrlDesc& D, const double* __restrict__ x0,
                                           const double* __restrict__ xref) {
-  extern __shared__ __align__(16) char smem[];
-  __shared__ TileScratch ts;
+  TileScratch& ts = tile_scratch();
   if (threadIdx.x == 0) mbar_init(&ts.mbar);
   __syncthreads();
   uint32_t phase = 0u;
-  run_tile_inl<MODEL, NPOS, false, SGF, GRID>(D, blockIdx.x, x0, xref, smem, ts, phase);
+  run_tile_inl<MODEL, NPOS, false, SGF, GRID>(D, blockIdx.x, x0, xref, phase);
 }
 
 }  // namespace dbm

@@ -97,18 +97,19 @@ struct HostOut {
 struct CtrlDesc {
   int model, K, T, J, P, n;
   int S, NPOS, nTiles, GT, nGroups;
-  float dt, h_eps, gamma_bas_f, R_B, C_coll, ln_mu, ln_sigma;
+  int nc;                    // far-field cells of a tile (far_cells), 0 = every pair directly
+  float r_body;              // largest distance of a shape point from the body's position
+  float dt, h_eps, C_coll, ln_mu, ln_sigma;
   float umin[2], umax[2];
   float Q[kMaxN], Qf[kMaxN];
   float shape[2 * kMaxShape];
   float g, inv_mass;
   float k_turn;              // arm / I (6-state quadrotor) or 1 / wheelbase (Ackermann)
   float inv_lambda_f;
-  double lambda, inv_lambda, mu_coarse, gamma_ctrl, gamma_bas, R_B_d;
+  double mu_coarse, gamma_bas, R_B_d;
   double umin_d[2], umax_d[2];
   int nscl;
   int sgf_wp;                // Savitzky-Golay window | order << 8, 0 = off (weights: cw)
-  double sigma[4];
   double Lsig[3];            // chol(Sigma): l00, l10, l11
   double Sinv[4];            // gamma * Sigma^-1 (row-major; zero when gamma = 0)
   double x_goal[kMaxN];
@@ -144,7 +145,7 @@ __host__ __device__ inline int sgf_table_offset(int T) { return (T + 3) & ~3; }
 // before the rollout, as the per-warp column sums of a merge and as the
 // nominal-rollout buffers in the final stage.
 struct SmemLayout {
-  int obs4, region, pose, V, red, Us, Usf, Uf, Af, colhi, collo, scl, xrf, shp, eS, cw, Sk, scH,
+  int obs4, cell, list, region, pose, V, red, Us, Usf, Uf, Af, colhi, collo, scl, xrf, shp, eS, cw, Sk, scH,
       scL, collf, xi, total;
 };
 
@@ -165,6 +166,67 @@ __host__ __device__ inline int merge_buf_bytes(int ncol, int nthreads) {
   return align_up(8 * merge_row_groups(ncol, nthreads) * (ncol + 1), 16);  // + Z
 }
 
+// ---- Far-field cells of the barrier.  A tile's (step, sample) units, in
+// step order, are cut into nc cells of consecutive units.  The poses of a
+// cell lie in a disc (centre p0, radius R, body included), and over that disc
+// the sum of 1 / h_j of the obstacles far from it is a smooth function: its
+// Taylor polynomial of degree kFarN about p0, built once per cell, replaces
+// one evaluation per point and obstacle.  The obstacles near the cell are
+// evaluated one by one as before.  With a_j = |p0 - c_j| - r_j the clearance
+// of the centre and t = R / a_j, the terms of degree n of 1 / h_j are at most
+// (n + 1) t^n / h_j(p0) anywhere in the disc, so the remainder is at most
+// (N + 2) t^(N+1) (1 + t)^2 / (1 - t)^2 of the term itself: 1.2e-7 (one FP32
+// rounding) at t = kFarRatio, reached only on the disc's rim by an obstacle at
+// the limit, and 2^-9 of that half way in.  A trajectory tile is small beside
+// the world: of 200 obstacles about 10 are near a cell of the 65536-sample
+// unicycle, of 500 about 40 near one of the crowded quadrotor.  Without and
+// with cells, a whole call: unicycle K 65536, T 100, J 200 608 and 365 us;
+// quadrotor K 32768, T 100, J 500, P 7 3090 and 830 us; vehicle K 9973, T 73,
+// J 117, P 8 305 and 162 us; 512 mixed controllers in one launch 29.2 and
+// 13.8 ms.  Degree 8 against 6 and 10, and cells of 1024 points against one or
+// sixteen per tile, come from counting the operations over the presets'
+// rollouts (least at 8 and 800 to 2800 points).
+constexpr int kFarN = 8;
+constexpr int kFarCoef = (kFarN + 1) * (kFarN + 2) / 2;
+constexpr float kFarRatio = 0.125f;
+constexpr int kFarMin = 12;       // fewer far obstacles than this cost less one by one
+constexpr int kFarMaxCells = 8;
+constexpr int kFarListMax = 512;  // near obstacles listed per cell at most
+struct __align__(16) FarCell {
+  float cx, cy, inv_R;
+  int n_near;               // obstacles listed, or -1: no polynomial, every obstacle directly
+  float2 c[kFarCoef + 1];   // coefficients in the order far_eval takes them, each twice
+};
+__host__ __device__ inline int far_list_cap(int J) {
+  const int c = J < kFarListMax ? J : kFarListMax;
+  return (c + 7) & ~7;
+}
+// Cells of a tile: about kFarCellPoints world points each (a cell's set-up
+// takes as long as evaluating some 50 points against every obstacle, and more
+// points make it wider), at most one per warp.  None where they would save too
+// little: in units of one point against one obstacle, a point costs J directly
+// and with cells about 9 (the polynomial), 8 + J / 10 near obstacles (what the
+// presets' densities give) and its share of the set-up.  The line of 4e7 over
+// the whole step is about 8 us of the GPU, what the last CTA's second look
+// (refine_samples) takes when it is needed: the quadrotor at K 4096, T 50,
+// J 40 (2e7) takes 71.5 us a call without cells, 72 to 80 us with them; at
+// K 8192, T 40, J 60 (7e7) 104 us without, 86 to 92 us with them.
+constexpr int kFarCellPoints = 1024;
+constexpr float kFarMinSaved = 4.0e7f;
+__host__ __device__ inline int far_cells(int K, int T, int S, int P, int J, int npos,
+                                         int nthreads) {
+  const int gsz = 32 * (npos / P);
+  const int groups = (T * S + gsz - 1) / gsz;
+  const int pts = T * S * P;
+  int nc = pts / kFarCellPoints;
+  if (nc > kFarMaxCells) nc = kFarMaxCells;
+  if (nc > nthreads / 32) nc = nthreads / 32;
+  if (nc > groups) nc = groups;
+  if (nc < 1) nc = 1;
+  const float setup = nc * (2800.0f + 53.0f * J) / pts;
+  return (float)K * T * P * (0.9f * J - 17.0f - setup) >= kFarMinSaved ? nc : 0;
+}
+
 // Row stride of the tile's (step, sample) arrays (poses, clamped controls,
 // unit sums): element (t, s) sits at t SP + s.  The rollout scans and the
 // per-sample cost loops step through a sample's row with lanes on
@@ -176,12 +238,16 @@ __host__ __device__ inline int merge_buf_bytes(int ncol, int nthreads) {
 __host__ __device__ inline int row_stride(int S, bool batched) { return batched ? (S | 1) : S; }
 
 __host__ __device__ inline SmemLayout smem_layout(int T, int S, int P, int J, int n, int nscl,
-                                                  int nwarps, bool batched) {
+                                                  int nwarps, int nc, bool batched) {
   SmemLayout L;
   int off = 0;
   L.obs4 = off;
   off += 16 * (J > 0 ? J : 1);
   off = align_up(off, 16);
+  L.cell = off;
+  off += nc * (int)sizeof(FarCell);
+  L.list = off;
+  off += align_up(2 * nc * far_list_cap(J), 16);
   L.region = off;
   const int SP = row_stride(S, batched);
   int main_b = 16 * T * SP + 8 * T * SP;
@@ -415,6 +481,14 @@ struct Dyn {
 };
 
 // ------------------------------------------------------------ tile kernel body
+// Weights of at least 1 / kRefShare are settled by direct sums
+// (refine_samples): at most kRefShare samples can have one.  Over two steps of
+// 84 problems U* then stays within 1e-5 of the direct evaluation's but for
+// three whose weights hang on the last bit of a cost; with 32 the first step's
+// largest differences are ten times those with 512, for 3 us less.
+constexpr int kRefShare = 128;
+constexpr int kRefMax = kRefShare + 8;
+static_assert(4 * kRefMax <= 8 * 4 * 32, "the list lies in the reduction scratch");
 struct TileScratch {
   uint64_t mbar;
   int flag;
@@ -424,6 +498,7 @@ struct TileScratch {
   double S_e_used, S_e_next;           // exploration rate of this step and the next
   unsigned long long iter;             // iteration counter of this step
   double x0[2];                        // measured position: origin of the tile's frame
+  int n_ref, n_tile;                   // samples whose costs the last CTA takes again (refine_list)
 };
 
 // The grid map as a tile reads it.  The tile's frame is centred on the
@@ -472,52 +547,243 @@ __device__ __forceinline__ float grid_h(const GridView& gv, float X, float Y) {
   return fmaf(fy, b - a, a);
 }
 
+// Minimum and maximum of a float over the warp, in one instruction each.
+__device__ __forceinline__ float warp_min_f(float v) {
+  float y;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(v));
+  return y;
+}
+__device__ __forceinline__ float warp_max_f(float v) {
+  float y;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(v));
+  return y;
+}
+
+// Place of unit u = t S + s in the tile's (step, sample) arrays: t SP + s =
+// u + (SP - S) floor(u / S), SP = row_stride(S, BATCHED); the quotient by one
+// multiply-high with m = ceil(2^32 / S), exact while u (m S - 2^32) < 2^32
+// (here u < T S <= 2^13 and m S - 2^32 < S <= 32).
+template <bool BATCHED>
+struct UnitIndex {
+  unsigned pad, mS;
+  __device__ __forceinline__ explicit UnitIndex(int S) {
+    pad = (unsigned)(row_stride(S, BATCHED) - S);
+    mS = pad ? 0xffffffffu / (unsigned)S + 1u : 0u;
+  }
+  __device__ __forceinline__ int operator()(int u) const {
+    if constexpr (BATCHED) return (int)((unsigned)u + pad * __umulhi((unsigned)u, mS));
+    else return u;
+  }
+};
+
+// Place of the coefficient of x^i y^k (i + k <= kFarN) in FarCell::c: Horner
+// in y from the highest power, inside it Horner in x from the highest power.
+__host__ __device__ constexpr int far_pos(int i, int k) {
+  return (kFarN - k) * (kFarN + 1 - k) / 2 + (kFarN - k - i);
+}
+
+// Set-up of one cell by one warp: the disc around the poses of units
+// [u0, u1), the obstacles near it (list, in order) and the Taylor
+// coefficients of the others' sum of 1 / h.  With D = p0 - c, H = |D|^2 - r^2
+// and d = R (x, y) the offset from p0,
+//   1 / h = 1 / (H + 2 D.d + |d|^2) = sum_n Q_n,  Q_0 = 1 / H,
+//   Q_{n+1} = -(2 D.d / H) Q_n - (|d|^2 / H) Q_{n-1},
+// the three-term recurrence of 1 / (1 - 2 x t + t^2); Q_n is homogeneous of
+// degree n, so its n + 1 coefficients follow from the two rows before.  Lanes
+// take obstacles; their sums are added across the warp with a transposing
+// butterfly (each lane ends with three of the coefficients).
+template <bool BATCHED>
+__device__ __noinline__ void far_setup(int cell_off, int list_off, int pose_off, int obs_off, int u0,
+                                       int u1, int S, int J, float r_body, float h_eps, int lane) {
+  extern __shared__ __align__(16) char smem[];
+  FarCell* cell = reinterpret_cast<FarCell*>(smem + cell_off);
+  unsigned short* list = reinterpret_cast<unsigned short*>(smem + list_off);
+  const float4* pose = reinterpret_cast<const float4*>(smem + pose_off);
+  const float4* obs4 = reinterpret_cast<const float4*>(smem + obs_off);
+  const int cap = far_list_cap(J);
+  const UnitIndex<BATCHED> at(S);
+  const float inf = __int_as_float(0x7f800000);
+  float x0 = inf, x1 = -inf, y0 = inf, y1 = -inf;
+  for (int u = u0 + lane; u < u1; u += 32) {
+    const float2 p = *reinterpret_cast<const float2*>(pose + at(u));
+    x0 = fminf(x0, p.x);
+    x1 = fmaxf(x1, p.x);
+    y0 = fminf(y0, p.y);
+    y1 = fmaxf(y1, p.y);
+  }
+  const float cx = 0.5f * (warp_min_f(x0) + warp_max_f(x1));
+  const float cy = 0.5f * (warp_min_f(y0) + warp_max_f(y1));
+  float m = 0.0f;
+  bool fine = true;  // every pose finite (and not so far that squares overflow)
+  for (int u = u0 + lane; u < u1; u += 32) {
+    const float2 p = *reinterpret_cast<const float2*>(pose + at(u));
+    const float dx = p.x - cx, dy = p.y - cy;
+    const float d2 = fmaf(dx, dx, dy * dy);
+    fine = fine && d2 < 1.0e30f;
+    m = fmaxf(m, d2);
+  }
+  const float R = (sqrt_approx(warp_max_f(m)) + r_body) * 1.00001f;
+  fine = __all_sync(0xffffffffu, fine);
+  // near obstacles: those whose clearance a is below R / kFarRatio, or whose h
+  // could come down to h_eps (h >= (a - R)^2 over the disc)
+  auto far = [&](int j, float& dx, float& dy, float& H) {
+    const float4 o = obs4[j];
+    dx = cx - o.x;
+    dy = cy - o.y;
+    const float d2 = fmaf(dx, dx, dy * dy);
+    H = fmaf(dx, dx, fmaf(dy, dy, o.z));
+    const float a = sqrt_approx(d2) - o.w, b = a - R;
+    return fine && R <= kFarRatio * a && b * b >= h_eps;
+  };
+  int nn = 0;
+  for (int j0 = 0; j0 < J; j0 += 32) {
+    const int j = j0 + lane;
+    float dx, dy, H;
+    const bool near = j < J && !far(j, dx, dy, H);
+    const unsigned b = __ballot_sync(0xffffffffu, near);
+    const int at_ = nn + __popc(b & ((1u << lane) - 1u));
+    if (near && at_ < cap) list[at_] = (unsigned short)j;
+    nn += __popc(b);
+  }
+  const bool direct = nn > cap || J - nn < kFarMin;
+  const float inv_R = R > 1.0e-30f ? 1.0f / R : 0.0f;
+  if (lane == 0) {
+    cell->cx = cx;
+    cell->cy = cy;
+    cell->inv_R = inv_R;
+    cell->n_near = direct ? -1 : nn;
+  }
+  if (direct) return;
+  float acc[48];
+#pragma unroll
+  for (int i = 0; i < 48; ++i) acc[i] = 0.0f;
+  for (int j = lane; j < J; j += 32) {
+    float dx, dy, H;
+    if (!far(j, dx, dy, H)) continue;
+    const float q = 1.0f / H, g = -2.0f * R * q;
+    const float ax = g * dx, ay = g * dy, b = -R * R * q;
+    float r0[kFarN + 1], r1[kFarN + 1];  // rows n - 1 and n
+    r0[0] = q;
+    r1[0] = ax * q;
+    r1[1] = ay * q;
+    acc[far_pos(0, 0)] += q;
+    acc[far_pos(1, 0)] += r1[0];
+    acc[far_pos(0, 1)] += r1[1];
+#pragma unroll
+    for (int n = 1; n < kFarN; ++n) {
+      float r2[kFarN + 1];
+#pragma unroll
+      for (int k = 0; k <= n + 1; ++k) {  // coefficient of x^(n+1-k) y^k
+        float v = k <= n ? ax * r1[k] : 0.0f;
+        if (k >= 1) v = k <= n ? fmaf(ay, r1[k - 1], v) : ay * r1[k - 1];
+        if (k <= n - 1) v = fmaf(b, r0[k], v);
+        if (k >= 2) v = fmaf(b, r0[k - 2], v);
+        r2[k] = v;
+        acc[far_pos(n + 1 - k, k)] += v;
+      }
+#pragma unroll
+      for (int k = 0; k <= n + 1; ++k) {
+        if (k <= n) r0[k] = r1[k];
+        r1[k] = r2[k];
+      }
+    }
+  }
+  __syncwarp();
+  int base = 0;
+#pragma unroll
+  for (int o = 16, n = 24; o >= 2; o >>= 1, n >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const float send = up ? acc[i] : acc[i + n];
+      const float keep = up ? acc[i + n] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    base += up ? n : 0;
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float v = acc[i] + __shfl_xor_sync(0xffffffffu, acc[i], 1);
+    if (!(lane & 1) && base + i < kFarCoef) cell->c[base + i] = make_float2(v, v);
+  }
+}
+
+// The far obstacles' sum of 1 / h at a thread's packed points: the cell's
+// polynomial by Horner's rule in two variables, 44 two-lane FMAs per pair of
+// points (as much as nine obstacles one by one).
+template <int NP2>
+__device__ __forceinline__ void far_eval(const FarCell* __restrict__ cell, const float2 (&X2)[NP2],
+                                         const float2 (&Y2)[NP2], float2 (&acc2)[NP2]) {
+  const float2 ncx = make_float2(-cell->cx, -cell->cx), ncy = make_float2(-cell->cy, -cell->cy);
+  const float2 ir = make_float2(cell->inv_R, cell->inv_R);
+  float2 x[NP2], y[NP2];
+#pragma unroll
+  for (int k = 0; k < NP2; ++k) {
+    x[k] = __fmul2_rn(__fadd2_rn(X2[k], ncx), ir);
+    y[k] = __fmul2_rn(__fadd2_rn(Y2[k], ncy), ir);
+    acc2[k] = cell->c[0];
+  }
+  int at = 1;
+#pragma unroll
+  for (int ky = kFarN - 1; ky >= 0; --ky) {
+    float2 r[NP2];
+    const float2 c0 = cell->c[at++];
+#pragma unroll
+    for (int k = 0; k < NP2; ++k) r[k] = c0;
+#pragma unroll
+    for (int i = kFarN - ky - 1; i >= 0; --i) {
+      const float2 c = cell->c[at++];
+#pragma unroll
+      for (int k = 0; k < NP2; ++k) r[k] = __ffma2_rn(r[k], x[k], c);
+    }
+#pragma unroll
+    for (int k = 0; k < NP2; ++k) acc2[k] = __ffma2_rn(acc2[k], y[k], r[k]);
+  }
+}
+
 // Fused barrier over nunits = T S (step, sample) units; unit u = t S + s has
 // its pose at pose[t SP + s] (SP = row_stride(S, BATCHED)) and P shape
-// points shp[0..P).  Each thread takes NPOS / P whole units at a
-// time (NPOS >= P), units base + k nthreads + tid (k < NPOS / P) so that
+// points shp[0..P).  A warp takes groups of 32 (NPOS / P) consecutive units
+// (NPOS >= P), each lane the units base + 32 k + lane (k < NPOS / P) so that
 // neighbouring lanes read neighbouring poses, keeps their world points in
-// registers and streams every
-// obstacle: h = |p - c|^2 - r^2 evaluated as fma(dx, dx, fma(dy, dy, -r^2)),
-// terms 1 / max(h, h_eps) added two obstacles at a time as (h1 + h2) / (h1 h2)
-// with the approximate reciprocal.  The points are held in packed pairs and
-// the subtractions, fmas, sums and products are packed two-lane FP32
-// instructions (each lane the same round-to-nearest operation as the scalar
-// one, so the results are the scalar loop's bit for bit): one issue slot
-// for two points, where the loop is bound by instruction issue.  A unit's
-// points are summed exactly (TwoSum) into (hi, lo), stored at
-// uB[u * ustride]; the sign bit of hi marks a unit in which some h <= 0
-// (collision).  A thread reads the poses of its units before it writes their
-// sums, so uB may overlay pose.  GRID: each point also adds the grid map's
-// term (grid_h) and counts its h in the collision test.
+// registers and streams the obstacles of the group's cell, or all of them
+// (nc = 0, or a cell without a polynomial): h = |p - c|^2 - r^2 evaluated as
+// fma(dx, dx, fma(dy, dy, -r^2)), terms 1 / max(h, h_eps) added two obstacles
+// at a time as (h1 + h2) / (h1 h2) with the approximate reciprocal.  The
+// points are held in packed pairs and the subtractions, fmas, sums and
+// products are packed two-lane FP32 instructions (each lane the same
+// round-to-nearest operation as the scalar one): one issue slot for two
+// points, where the loop is bound by instruction issue.  A unit's points
+// are summed exactly (TwoSum) into (hi, lo), stored at uB[u * ustride]; the
+// sign bit of hi marks a unit in which some h <= 0 (collision; a far obstacle
+// has h >= h_eps all over its cell).  A lane reads the poses of its units
+// before it writes their sums, so uB may overlay pose.  GRID: each point also
+// adds the grid map's term (grid_h) and counts its h in the collision test.
 template <int NPOS, bool BATCHED, bool GRID = false>
 __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, const float4* pose,
                                               const float2* __restrict__ shp,
                                               const float4* __restrict__ obs4, float h_eps,
-                                              float2* uB, int ustride, int tid, int nthreads,
+                                              float2* uB, int ustride, int tid, int nthreads, int nc,
+                                              const FarCell* __restrict__ cells,
+                                              const unsigned short* __restrict__ lists,
                                               const GridView* gv = nullptr) {
-  // unit u = t S + s lives at t SP + s = u + (SP - S) floor(u / S); the
-  // quotient by one multiply-high with m = ceil(2^32 / S), exact while
-  // u (m S - 2^32) < 2^32 (here u < T S <= 2^13 and m S - 2^32 < S <= 32)
-  const unsigned pad = (unsigned)(row_stride(S, BATCHED) - S);
-  const unsigned mS = pad ? 0xffffffffu / (unsigned)S + 1u : 0u;
-  auto at = [&](int u) {
-    if constexpr (BATCHED) return (int)((unsigned)u + pad * __umulhi((unsigned)u, mS));
-    else return u;
-  };
+  const UnitIndex<BATCHED> at(S);
   static_assert(NPOS % 2 == 0, "points are held in packed pairs");
   constexpr int NP2 = NPOS / 2;
-  const int upt = NPOS / P;  // units per thread per round
+  const int upt = NPOS / P;  // units per lane
   const int used = upt * P;
-  for (int ub = tid; ub < nunits; ub += nthreads * upt) {  // ub: this round's first unit
+  const int lane = tid & 31, nwarps = nthreads >> 5;
+  const int gsz = 32 * upt, NG = (nunits + gsz - 1) / gsz;
+  for (int g = tid >> 5; g < NG; g += nwarps) {
+    const int ub = g * gsz + lane;  // this lane's first unit
     float2 X2[NP2], Y2[NP2], acc2[NP2];  // points 2k and 2k + 1
     float mn[NPOS];
     int uu = 0, p = 0;
 #pragma unroll
     for (int i = 0; i < NPOS; ++i) {
-      const int u = ub + uu * nthreads;
+      const int u = ub + uu * 32;
       const bool ok = (i < used) && (u < nunits);
-      const float4 ps = pose[at(ok ? u : ub)];
+      const float4 ps = pose[at(ok ? u : nunits - 1)];
       const float2 sh = shp[ok ? p : 0];
       const float X = fmaf(ps.z, sh.x, fmaf(-ps.w, sh.y, ps.x));
       const float Y = fmaf(ps.w, sh.x, fmaf(ps.z, sh.y, ps.y));
@@ -536,34 +802,7 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
     }
 #pragma unroll
     for (int k = 0; k < NP2; ++k) acc2[k] = make_float2(0.0f, 0.0f);
-    // obstacles in pairs: 1/h1 + 1/h2 = (h1 + h2) / (h1 h2), one reciprocal
-    // for two terms (h1 h2 stays finite for |p - c| < 4e9 m and h_eps >= 1e-18);
-    // with more points per thread the pair's temporaries would not fit
-    int j = 0;
-    if constexpr (NPOS <= 8)
-    for (; j + 1 < J; j += 2) {
-      const float4 o = obs4[j], q = obs4[j + 1];
-      const float2 nox = make_float2(-o.x, -o.x), noy = make_float2(-o.y, -o.y);
-      const float2 noz = make_float2(o.z, o.z);
-      const float2 nqx = make_float2(-q.x, -q.x), nqy = make_float2(-q.y, -q.y);
-      const float2 nqz = make_float2(q.z, q.z);
-#pragma unroll
-      for (int k = 0; k < NP2; ++k) {
-        const float2 dx = __fadd2_rn(X2[k], nox), dy = __fadd2_rn(Y2[k], noy);
-        const float2 ex = __fadd2_rn(X2[k], nqx), ey = __fadd2_rn(Y2[k], nqy);
-        float2 h1 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, noz));
-        float2 h2 = __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, nqz));
-        mn[2 * k] = fmin3(mn[2 * k], h1.x, h2.x);
-        mn[2 * k + 1] = fmin3(mn[2 * k + 1], h1.y, h2.y);
-        h1 = make_float2(fmaxf(h1.x, h_eps), fmaxf(h1.y, h_eps));
-        h2 = make_float2(fmaxf(h2.x, h_eps), fmaxf(h2.y, h_eps));
-        const float2 pr = __fmul2_rn(h1, h2);
-        const float2 r = make_float2(rcp_approx(pr.x), rcp_approx(pr.y));
-        acc2[k] = __ffma2_rn(__fadd2_rn(h1, h2), r, acc2[k]);
-      }
-    }
-    for (; j < J; ++j) {
-      const float4 o = obs4[j];
+    auto one = [&](const float4 o) {
       const float2 nox = make_float2(-o.x, -o.x), noy = make_float2(-o.y, -o.y);
       const float2 noz = make_float2(o.z, o.z);
 #pragma unroll
@@ -575,6 +814,50 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
         acc2[k] = __fadd2_rn(acc2[k], make_float2(rcp_approx(fmaxf(h.x, h_eps)),
                                                   rcp_approx(fmaxf(h.y, h_eps))));
       }
+    };
+    // obstacles in pairs: 1/h1 + 1/h2 = (h1 + h2) / (h1 h2), one reciprocal
+    // for two terms (h1 h2 stays finite for |p - c| < 4e9 m and h_eps >= 1e-18);
+    // with more points per thread the pair's temporaries would not fit
+    auto two = [&](const float4 o, const float4 q) {
+      if constexpr (NPOS <= 8) {
+        const float2 nox = make_float2(-o.x, -o.x), noy = make_float2(-o.y, -o.y);
+        const float2 noz = make_float2(o.z, o.z);
+        const float2 nqx = make_float2(-q.x, -q.x), nqy = make_float2(-q.y, -q.y);
+        const float2 nqz = make_float2(q.z, q.z);
+#pragma unroll
+        for (int k = 0; k < NP2; ++k) {
+          const float2 dx = __fadd2_rn(X2[k], nox), dy = __fadd2_rn(Y2[k], noy);
+          const float2 ex = __fadd2_rn(X2[k], nqx), ey = __fadd2_rn(Y2[k], nqy);
+          float2 h1 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, noz));
+          float2 h2 = __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, nqz));
+          mn[2 * k] = fmin3(mn[2 * k], h1.x, h2.x);
+          mn[2 * k + 1] = fmin3(mn[2 * k + 1], h1.y, h2.y);
+          h1 = make_float2(fmaxf(h1.x, h_eps), fmaxf(h1.y, h_eps));
+          h2 = make_float2(fmaxf(h2.x, h_eps), fmaxf(h2.y, h_eps));
+          const float2 pr = __fmul2_rn(h1, h2);
+          const float2 r = make_float2(rcp_approx(pr.x), rcp_approx(pr.y));
+          acc2[k] = __ffma2_rn(__fadd2_rn(h1, h2), r, acc2[k]);
+        }
+      } else {
+        one(o);
+        one(q);
+      }
+    };
+    const int c = nc > 0 ? g * nc / NG : 0;
+    int nn = nc > 0 ? cells[c].n_near : -1;
+    if (nn >= 0) {
+      far_eval<NP2>(cells + c, X2, Y2, acc2);
+      const unsigned short* l = lists + c * far_list_cap(J);
+      int j = 0;
+      for (; j + 1 < nn; j += 2) {
+        const unsigned jj = *reinterpret_cast<const unsigned*>(l + j);
+        two(obs4[jj & 0xffffu], obs4[jj >> 16]);
+      }
+      if (j < nn) one(obs4[l[j]]);
+    } else {
+      int j = 0;
+      for (; j + 1 < J; j += 2) two(obs4[j], obs4[j + 1]);
+      if (j < J) one(obs4[j]);
     }
     if constexpr (GRID) {
       if (gv->g) {
@@ -592,13 +875,14 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
     bool coll = false;
     uu = 0;
     p = 0;
+    __syncwarp();
 #pragma unroll
     for (int i = 0; i < NPOS; ++i) {
       if (i < used) {
         ff_add(f, (i & 1) ? acc2[i >> 1].y : acc2[i >> 1].x);
         coll |= (mn[i] <= 0.0f);
         if (++p == P) {
-          const int u = ub + uu * nthreads;
+          const int u = ub + uu * 32;
           if (u < nunits) uB[(size_t)at(u) * ustride] = make_float2(coll ? -f.hi : f.hi, f.lo);
           f.hi = 0.0f;
           f.lo = 0.0f;
@@ -607,6 +891,85 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
           ++uu;
         }
       }
+    }
+  }
+}
+
+// The barrier of a few samples (Sc of them, their poses at pose[t SP + s]),
+// every obstacle directly, with the points spread over the lanes: the points
+// of a unit on 1, 2, 4 or 8 neighbouring lanes, two units per lane as a packed
+// pair.  Each point's sum and each unit's sum are formed by the operations of
+// barrier_units without cells, in the same order, so they are the same bits.
+// For the last CTA of a step, which runs it alone: the time is that of one
+// lane's loop over the obstacles.
+template <int NPOS, bool GRID>
+__device__ __forceinline__ void barrier_refine(int Sc, int T, int SP, int P, int J,
+                                               const float4* pose, const float2* __restrict__ shp,
+                                               const float4* __restrict__ obs4, float h_eps,
+                                               float2* uB, int ustride, int tid, int nthreads,
+                                               const GridView* gv) {
+  const int lp = P <= 1 ? 1 : P <= 2 ? 2 : P <= 4 ? 4 : 8;  // lanes per unit
+  const int lane = tid & 31, upw = 32 / lp, p = lane & (lp - 1), first = lane - p;
+  const int nunits = Sc * T;
+  const float2 sh = shp[min(p, P - 1)];
+  for (int u0 = (tid >> 5) * 2 * upw; u0 < nunits; u0 += (nthreads >> 5) * 2 * upw) {
+    int at[2];
+    float2 X, Y, acc = make_float2(0.0f, 0.0f);
+    float mn[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int u = min(u0 + q * upw + lane / lp, nunits - 1);
+      const int t = u / Sc;
+      at[q] = t * SP + (u - t * Sc);
+      const float4 ps = pose[at[q]];
+      (q ? X.y : X.x) = fmaf(ps.z, sh.x, fmaf(-ps.w, sh.y, ps.x));
+      (q ? Y.y : Y.x) = fmaf(ps.w, sh.x, fmaf(ps.z, sh.y, ps.y));
+      mn[q] = __int_as_float(0x7f800000);
+    }
+    auto h_of = [&](const float4 o) {
+      const float2 dx = __fadd2_rn(X, make_float2(-o.x, -o.x)), dy = __fadd2_rn(Y, make_float2(-o.y, -o.y));
+      return __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, make_float2(o.z, o.z)));
+    };
+    int j = 0;
+    if constexpr (NPOS <= 8) {
+#pragma unroll 2
+      for (; j + 1 < J; j += 2) {
+        float2 h1 = h_of(obs4[j]), h2 = h_of(obs4[j + 1]);
+        mn[0] = fmin3(mn[0], h1.x, h2.x);
+        mn[1] = fmin3(mn[1], h1.y, h2.y);
+        h1 = make_float2(fmaxf(h1.x, h_eps), fmaxf(h1.y, h_eps));
+        h2 = make_float2(fmaxf(h2.x, h_eps), fmaxf(h2.y, h_eps));
+        const float2 pr = __fmul2_rn(h1, h2);
+        acc = __ffma2_rn(__fadd2_rn(h1, h2), make_float2(rcp_approx(pr.x), rcp_approx(pr.y)), acc);
+      }
+    }
+#pragma unroll 4
+    for (; j < J; ++j) {
+      const float2 h = h_of(obs4[j]);
+      mn[0] = fminf(mn[0], h.x);
+      mn[1] = fminf(mn[1], h.y);
+      acc = __fadd2_rn(acc, make_float2(rcp_approx(fmaxf(h.x, h_eps)), rcp_approx(fmaxf(h.y, h_eps))));
+    }
+    if constexpr (GRID) {
+      if (gv->g) {
+        const float hx = grid_h(*gv, X.x, Y.x), hy = grid_h(*gv, X.y, Y.y);
+        mn[0] = fminf(mn[0], hx);
+        mn[1] = fminf(mn[1], hy);
+        acc = __fadd2_rn(acc, make_float2(rcp_approx(fmaxf(hx, h_eps)), rcp_approx(fmaxf(hy, h_eps))));
+      }
+    }
+    __syncwarp();
+    FF f[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+    for (int i = 0; i < P; ++i) {
+      ff_add(f[0], __shfl_sync(0xffffffffu, acc.x, first + i));
+      ff_add(f[1], __shfl_sync(0xffffffffu, acc.y, first + i));
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const unsigned hit = __ballot_sync(0xffffffffu, mn[q] <= 0.0f);
+      const bool coll = (hit >> first) & ((1u << lp) - 1u);
+      if (p == 0 && u0 + q * upw + lane / lp < nunits)
+        uB[(size_t)at[q] * ustride] = make_float2(coll ? -f[q].hi : f[q].hi, f[q].lo);
     }
   }
 }

@@ -400,6 +400,23 @@ __device__ __forceinline__ GridView grid_view(const CtrlDesc& D, const double* _
   return gv;
 }
 
+// The CTA's shared memory, named where it is used.  The tile functions that
+// are called out of line would otherwise get it as generic pointers, whose
+// loads and stores are slower than those of the shared window.
+__device__ __forceinline__ char* dyn_smem() {
+  extern __shared__ __align__(16) char smem[];
+  return smem;
+}
+__device__ __forceinline__ TileScratch& tile_scratch() {
+  __shared__ TileScratch s;
+  return s;
+}
+// The persistent kernels' copy of the descriptor of the tile at hand.
+__device__ __forceinline__ CtrlDesc& tile_desc() {
+  __shared__ CtrlDesc s;
+  return s;
+}
+
 // The CTA's copy of its grid view (only the grid kernels instantiate it).
 __device__ __forceinline__ GridView& grid_shared() {
   __shared__ GridView s;
@@ -447,7 +464,8 @@ __device__ __forceinline__ void sgf_columns(const float* __restrict__ w, int W, 
 // (that costs another barrier and more code, which a step run after an L2
 // flush fetches from memory).
 template <int MODEL, int NPOS, bool GRID = false>
-__device__ void final_stage(const CtrlDesc& D, char* smem, const SmemLayout& L, TileScratch& ts,
+__device__ __forceinline__ void final_stage(const CtrlDesc& D, char* smem, const SmemLayout& L,
+                                            TileScratch& ts,
                             double* out, const GridView* gv = nullptr) {
   const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int T = D.T, P = D.P;
@@ -564,6 +582,161 @@ __device__ void final_stage(const CtrlDesc& D, char* smem, const SmemLayout& L, 
   }
 }
 
+// The samples that hold at least 1 / kRefShare of the normaliser Z, at most
+// kRefShare of them: into ref_k, ascending.  Called by the last CTA after
+// the last merge, whose source scales (the tiles', or with two levels the
+// groups') scl holds; the tiles' minima and then the costs of the few tiles
+// that can hold one are read again.  Scratch: ref_tile (kRefMax ints).
+constexpr int kRefPer = (kRefMax + 63) / 64;  // list entries per thread at most
+__device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, const float* scl,
+                                            int* ref_k, int* ref_tile, int tid, int nthreads) {
+  const int lane = tid & 31;
+  const float zmin = ts.Z.hi / kRefShare, tmin = 0.9999f * zmin;
+  if (tid == 0) ts.n_ref = ts.n_tile = 0;
+  __syncthreads();
+  for (int i = tid; i < D.nTiles; i += nthreads) {
+    float sc = scl[D.nGroups > 1 ? i / D.GT : i];
+    if (D.nGroups > 1 && sc >= tmin)
+      sc = expf(-(__ldcg(&D.part_rz[i].x) - ts.ref) * D.inv_lambda_f);
+    if (sc >= tmin) {
+      const int at = atomicAdd(&ts.n_tile, 1);
+      if (at < kRefMax) ref_tile[at] = i;
+    }
+  }
+  __syncthreads();
+  const double base = ts.base, ref = (double)ts.ref;
+  const int n_tile = min(ts.n_tile, kRefMax);
+  for (int q = tid >> 5; q < n_tile; q += nthreads >> 5) {
+    const int k = ref_tile[q] * D.S + lane;
+    if (lane < D.S && k < D.K) {
+      const float e = expf(-(float)(__ldcg(D.costs + k) - base - ref) * D.inv_lambda_f);
+      if (e >= zmin) {
+        const int at = atomicAdd(&ts.n_ref, 1);
+        if (at < kRefMax) ref_k[at] = k;
+      }
+    }
+  }
+  __syncthreads();
+  // in ascending order: the sums do not depend on who came first
+  const int n = min(ts.n_ref, kRefMax);
+  int v[kRefPer], r[kRefPer];
+#pragma unroll
+  for (int q = 0; q < kRefPer; ++q) {
+    const int i = tid + q * nthreads;
+    v[q] = i < n ? ref_k[i] : 0x7fffffff;
+    r[q] = 0;
+    if (i < n)
+      for (int j = 0; j < n; ++j) r[q] += ref_k[j] < v[q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kRefPer; ++q)
+    if (tid + q * nthreads < n) ref_k[r[q]] = v[q];
+  if (tid == 0) ts.n_ref = n;
+  __syncthreads();
+}
+
+// Second look at the samples that carry the weights, after the last merge of
+// a step whose tiles used far-field cells: their costs once more with every
+// obstacle summed directly, and the change of their weights put into Z and
+// the merged column sums.  A weight is the exponential of a cost difference,
+// so where a few samples share all of it the rounding of their costs goes
+// straight into U*: some 1e-5 of a barrier cost of hundreds, whichever way it
+// is summed.  Taking those few again leaves the polynomial no say in it: they
+// end with the bits of the direct evaluation.  They are drawn and rolled out
+// anew (the generator is counter based).  The last CTA runs this alone, a
+// chain of latencies (about 8 us); out of line, so that its registers leave
+// the tile's code as it is.
+template <int MODEL, int NPOS, bool BATCHED, bool GRID>
+__device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
+  const CtrlDesc& D = BATCHED ? tile_desc() : D_;
+  char* smem = dyn_smem();
+  TileScratch& ts = tile_scratch();
+  const int tid = threadIdx.x, nthreads = blockDim.x;
+  const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
+  const int T = D.T, P = D.P, J = D.J;
+  const SmemLayout L = smem_layout(T, D.S, P, J, Dyn<MODEL>::n, D.nscl, nwarps, D.nc, BATCHED);
+  int* ref_k = reinterpret_cast<int*>(smem + L.red);
+  refine_list(D, ts, reinterpret_cast<const float*>(smem + L.scl), ref_k,
+              reinterpret_cast<int*>(smem + L.region), tid, nthreads);
+  const float2* Uf = reinterpret_cast<const float2*>(smem + L.Uf);
+  const float* cw = reinterpret_cast<const float*>(smem + L.cw);
+  float* eS = reinterpret_cast<float*>(smem + L.eS);
+  float* scH = reinterpret_cast<float*>(smem + L.scH);
+  float* scL = reinterpret_cast<float*>(smem + L.scL);
+  float* col_hi = reinterpret_cast<float*>(smem + L.colhi);
+  float* col_lo = reinterpret_cast<float*>(smem + L.collo);
+  float4* pose = reinterpret_cast<float4*>(smem + L.region);
+  const float2* uB = reinterpret_cast<const float2*>(pose);
+  const DevState* st = D.st;
+  const uint32_t it_lo = (uint32_t)(ts.iter & 0xffffffffull), it_hi = (uint32_t)(ts.iter >> 32);
+  const int n_ref = ts.n_ref;
+  for (int r0 = 0; r0 < n_ref; r0 += D.S) {
+    const int Sc = min(D.S, n_ref - r0);
+    float2* V = reinterpret_cast<float2*>(pose + T * Sc);
+    for (int i = tid; i < T * Sc; i += nthreads) {
+      const int t = i / Sc, s = i - t * Sc;
+      const uint4 r = philox4x32_10(make_uint4((uint32_t)ref_k[r0 + s], (uint32_t)t, it_lo, it_hi),
+                                    D.key0, D.key1);
+      const float2 du = nln_draw(r, st->L00, st->L10, st->L11, D.ln_mu, D.ln_sigma), u = Uf[t];
+      V[i] = make_float2(fminf(fmaxf(u.x + du.x, D.umin[0]), D.umax[0]),
+                         fminf(fmaxf(u.y + du.y, D.umin[1]), D.umax[1]));
+    }
+    __syncthreads();
+    for (int s = warp; s < Sc; s += nwarps) {
+      FF c = {0.0f, 0.0f};
+      scan_trajectory<MODEL, true>(D, T, V + s, Sc, reinterpret_cast<const float*>(smem + L.xi),
+                                   pose + s, Sc, Uf, reinterpret_cast<const float2*>(smem + L.Af),
+                                   reinterpret_cast<const float*>(smem + L.xrf), c, lane);
+      c = warp_sum_ff(c);
+      if (lane == 0) {
+        scH[s] = c.hi;
+        scL[s] = c.lo;
+      }
+    }
+    __syncthreads();
+    barrier_refine<NPOS, GRID>(Sc, T, Sc, P, J, pose, reinterpret_cast<const float2*>(smem + L.shp),
+                               reinterpret_cast<const float4*>(smem + L.obs4), D.h_eps,
+                               reinterpret_cast<float2*>(pose), 2, tid, nthreads,
+                               GRID ? &grid_shared() : nullptr);
+    __syncthreads();
+    for (int s = warp; s < Sc; s += nwarps) {
+      const int k = ref_k[r0 + s];
+      const double was = __ldcg(D.costs + k) - ts.base;
+      FF b = {0.0f, 0.0f};
+      for (int t = lane; t < T; t += 32) {
+        const float2 v = uB[2 * (t * Sc + s)];
+        ff_add_prod(b, cw[t], fabsf(v.x), v.y);
+        if (__float_as_int(v.x) < 0) ff_add(b, D.C_coll);
+      }
+      __syncwarp();
+      b = warp_sum_ff(b);
+      if (lane == 0) {
+        const FF c = ff_norm(ff_sum(FF{scH[s], scL[s]}, b));
+        const double now = (double)c.hi + (double)c.lo;
+        D.costs[k] = ts.base + now;
+        eS[s] = expf(-(float)(now - (double)ts.ref) * D.inv_lambda_f) -
+                expf(-(float)(was - (double)ts.ref) * D.inv_lambda_f);
+      }
+    }
+    __syncthreads();
+    for (int c = tid; c < 2 * T; c += nthreads) {
+      const float* Vt = reinterpret_cast<const float*>(V + (c >> 1) * Sc) + (c & 1);
+      const float u = reinterpret_cast<const float*>(Uf)[c];
+      FF a = {col_hi[c], col_lo[c]};
+      for (int s = 0; s < Sc; ++s) ff_add(a, eS[s] * (Vt[2 * s] - u));
+      col_hi[c] = a.hi;
+      col_lo[c] = a.lo;
+    }
+    if (tid == 0) {
+      FF z = ts.Z;
+      for (int s = 0; s < Sc; ++s) ff_add(z, eS[s]);
+      ts.Z = ff_norm(z);
+    }
+    __syncthreads();
+  }
+}
+
 // One tile of one controller.  ts.mbar must be initialised; mbar_phase is
 // each thread's own copy of the parity of the barrier's next completion.
 // BATCHED: the tile runs in the persistent batch kernel, which takes the
@@ -583,15 +756,16 @@ __device__ void final_stage(const CtrlDesc& D, char* smem, const SmemLayout& L, 
 template <int MODEL, int NPOS, bool BATCHED, bool SGF = BATCHED, bool GRID = false>
 __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
                                              const double* __restrict__ x0g,
-                                             const double* __restrict__ xrefg, char* smem,
-                                             TileScratch& ts, uint32_t& mbar_phase,
+                                             const double* __restrict__ xrefg, uint32_t& mbar_phase,
                                              double* u0_out = nullptr) {
+  char* smem = dyn_smem();
+  TileScratch& ts = tile_scratch();
   constexpr int n = Dyn<MODEL>::n;
   const int tid = threadIdx.x, nthreads = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
   const int T = D.T, S = D.S, P = D.P, J = D.J, K = D.K;
   const int SP = row_stride(S, BATCHED);  // row stride of the (t, s) arrays
-  const SmemLayout L = smem_layout(T, S, P, J, n, D.nscl, nwarps, BATCHED);
+  const SmemLayout L = smem_layout(T, S, P, J, n, D.nscl, nwarps, D.nc, BATCHED);
   float4* obs4 = reinterpret_cast<float4*>(smem + L.obs4);
   float4* pose = reinterpret_cast<float4*>(smem + L.pose);
   float2* uB = reinterpret_cast<float2*>(smem + L.pose);  // overlays pose, stride 2
@@ -682,7 +856,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
     // the raw (region) and converted (obs4) areas are distinct
     for (int j = tid; j < J; j += nthreads) {
       double cx = raw[3 * j], cy = raw[3 * j + 1], r = raw[3 * j + 2];
-      obs4[j] = make_float4((float)(cx - ox), (float)(cy - oy), -(float)(r * r), 0.0f);
+      obs4[j] = make_float4((float)(cx - ox), (float)(cy - oy), -(float)(r * r), (float)r);
     }
   }
   __syncthreads();
@@ -780,13 +954,30 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
   }
   __syncthreads();
 
+  // ---- far-field cells: one warp sets up one cell of the tile's units
+  FarCell* cells = reinterpret_cast<FarCell*>(smem + L.cell);
+  unsigned short* lists = reinterpret_cast<unsigned short*>(smem + L.list);
+  const int nc = D.nc;
+  if (nc > 0) {
+    if (warp < nc) {
+      const int gsz = 32 * (NPOS / P), NG = (T * S + gsz - 1) / gsz;
+      // the groups g of cell c are those with g nc / NG = c
+      const int g0 = (warp * NG + nc - 1) / nc, g1 = ((warp + 1) * NG + nc - 1) / nc;
+      far_setup<BATCHED>(L.cell + warp * (int)sizeof(FarCell), L.list + 2 * warp * far_list_cap(J),
+                         L.pose, L.obs4, g0 * gsz, min(g1 * gsz, T * S), S, J, D.r_body, D.h_eps,
+                         lane);
+    }
+    __syncthreads();
+  }
+
   // ---- fused barrier over all (step, sample) units, sums over the poses
   if constexpr (GRID) {
     const GridView gv = grid_shared();
     barrier_units<NPOS, BATCHED, true>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid,
-                                       nthreads, &gv);
+                                       nthreads, nc, cells, lists, &gv);
   } else {
-    barrier_units<NPOS, BATCHED>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid, nthreads);
+    barrier_units<NPOS, BATCHED>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid, nthreads,
+                                 nc, cells, lists);
   }
   __syncthreads();
 
@@ -901,6 +1092,9 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
                              D.inv_lambda_f, scl, zi, mbuf, &ts.ref, &ts.Z, col_hi, col_lo, tid,
                              nthreads);
   }
+  // (one sample with all but 1 / kRefShare of the weight needs no second look)
+  if (nc > 0 && ts.Z.hi > 1.0f + 1.0f / kRefShare)
+    refine_samples<MODEL, NPOS, BATCHED, GRID>(D);
   if constexpr (SGF) {
     if (D.sgf_wp)
       sgf_columns(D.cw + sgf_table_offset(T), D.sgf_wp & 0xff, T, col_hi, col_lo,
@@ -915,12 +1109,12 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
   }
 }
 
-template <int MODEL, int NPOS, bool BATCHED, bool SGF = BATCHED, bool GRID = false>
-__device__ __noinline__ void run_tile(const CtrlDesc& D, int tile, const double* __restrict__ x0g,
-                                      const double* __restrict__ xrefg, char* smem,
-                                      TileScratch& ts, uint32_t& mbar_phase,
-                                      double* u0_out = nullptr) {
-  run_tile_inl<MODEL, NPOS, BATCHED, SGF, GRID>(D, tile, x0g, xrefg, smem, ts, mbar_phase, u0_out);
+// The tile of the persistent kernels, whose descriptor is tile_desc().
+template <int MODEL, int NPOS>
+__device__ __noinline__ void run_tile(int tile, const double* __restrict__ x0g,
+                                      const double* __restrict__ xrefg, uint32_t& mbar_phase,
+                                      double* u0_out) {
+  run_tile_inl<MODEL, NPOS, true>(tile_desc(), tile, x0g, xrefg, mbar_phase, u0_out);
 }
 
 }  // namespace dbm
