@@ -386,9 +386,40 @@ void free_ctx(mppi_ctx* c) {
   delete c;
 }
 
-// Launch shape: S samples per CTA, chosen so the grid covers the SMs at
-// least twice when K allows, then shrunk until the tile's shared memory
-// (whole-horizon poses and controls, obstacles) fits.
+// Launch shape, where the caller leaves it open: S samples per CTA and the
+// threads of a CTA, by K alone, then S shrunk until the tile's shared memory
+// (whole-horizon poses and controls, obstacles) fits.  Measured over ten
+// problems, every S from 1 to 32 at 128, 256 and 512 threads (us a step in a
+// row, against two CTAs of 256 threads per SM with S up to 32):
+//  - up to 32 samples per SM, one CTA of 512 threads on each: the step is one
+//    tile's chain of phases and the merge of its rows, so the fewest rows (one
+//    merge level) and the most warps win (quadrotor K 4096 48.1 -> 44.3,
+//    K 1024 33.6 -> 28.9, smoothed K 1024 22.7 -> 20.8, unicycle K 4096
+//    26.7 -> 24.6).  At least 5 samples: of a smaller tile the merge is the
+//    longer part; below 7, 256 threads (unicycle K 256 20.6 -> 16.6);
+//  - up to 64, two CTAs of 256 threads on each SM, up to 96 three, still one
+//    wave (vehicle K 9973, T 73 132 -> 103; the quadrotor at K 8192 takes 57.6
+//    with two and 56.6 with three, but 70 and 73 a call with host inputs,
+//    which every CTA reads over the host link);
+//  - beyond, several waves of 31 (unicycle K 65536 335 -> 286, quadrotor
+//    K 32768 707 -> 684).
+// From 12 on, S avoids multiples of 4: the scans read a sample's steps S
+// words of 8 or 16 bytes apart, and those strides fold the lanes onto a few
+// shared-memory banks (S 32 against 31 is the unicycle's 335 against 286).
+constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31;
+void default_shape(int K, int sms, int* S, int* threads) {
+  if (K <= 32 * sms) {
+    *S = std::max(kTileMin, (K + sms - 1) / sms);
+    *threads = *S >= kTileWide ? 512 : 256;
+  } else {
+    const int per_sm = K <= 64 * sms ? 2 : 3;
+    *S = K <= 96 * sms ? (K + per_sm * sms - 1) / (per_sm * sms) : kTileLarge;
+    *threads = 256;
+  }
+  if (*S >= 12 && *S % 4 == 0) *S += *S < 32 ? 1 : -1;
+  *S = std::min(*S, K);
+}
+
 int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tiling* out,
                   int* smem_out, int* nc_out, bool batched = false) {
   const int sms = num_sms();
@@ -397,8 +428,16 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
   if (req) t = *req;
   const bool fixed_S = t.samples_per_cta > 0;
   if (!fixed_S) {
-    long want = ((long)p->K + 2L * sms - 1) / (2L * sms);
-    t.samples_per_cta = (int)(want < 1 ? 1 : (want > 32 ? 32 : want));
+    int threads = 0;
+    default_shape(p->K, sms, &t.samples_per_cta, &threads);
+    if (t.threads <= 0) t.threads = threads;
+    // a context takes its obstacles later: tiles larger than two per SM make
+    // leave room for the largest set
+    const int two = std::min(32, (p->K + 2 * sms - 1) / (2 * sms));
+    while (t.samples_per_cta > two &&
+           smem_layout(p->T, t.samples_per_cta, p->n_shape, MPPI_MAX_OBSTACLES, n, 256,
+                       t.threads / 32, 0, batched).total > max_smem_optin())
+      --t.samples_per_cta;
   }
   if (t.samples_per_cta > 32) return fail(MPPI_EINVAL, "samples_per_cta must be <= 32");
   if (t.threads <= 0) t.threads = 256;
@@ -1079,33 +1118,43 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   mppi_ctx c;  // on the stack: only its descriptor logic is used
   c.p = *p;
   c.n = state_dim(p->model);
-  rc = choose_tiling(p, nullptr, J, &c.tl, &c.smem, &c.nc);
-  if (rc) return rc;
   const int T = p->T, K = p->K;
-  const int nTiles = (K + c.tl.samples_per_cta - 1) / c.tl.samples_per_cta;
-  const int GT = group_size(nTiles);
-  const int nGroups = (nTiles + GT - 1) / GT;
+  int nTiles = 0, nGroups = 0;
+  size_t off = 0, o_st, o_cU, o_cA, o_cw, o_obst, o_part, o_prz, o_gpart, o_grz, o_cnt, o_costs,
+      o_coll, o_Ustar;
+  // the library's launch shape, or tiles of 32 (the fewest rows) where its
+  // partial rows do not fit the scratch
+  const mppi_tiling largest = {32, 256, 0, 0};
+  for (const mppi_tiling* req : {(const mppi_tiling*)nullptr, &largest}) {
+    rc = choose_tiling(p, req, J, &c.tl, &c.smem, &c.nc);
+    if (rc && req) break;  // off is still the first shape's, above the limit
+    if (rc) return rc;
+    nTiles = (K + c.tl.samples_per_cta - 1) / c.tl.samples_per_cta;
+    const int GT = group_size(nTiles);
+    nGroups = (nTiles + GT - 1) / GT;
+    off = 0;
+    o_st = carve(&off, sizeof(DevState));
+    o_cU = carve(&off, sizeof(float2) * T);
+    o_cA = carve(&off, sizeof(float2) * T);
+    o_cw = carve(&off, cw_bytes(p));
+    o_obst = carve(&off, (size_t)align_up(24 * (J > 0 ? J : 1), 16));
+    o_part = carve(&off, sizeof(float) * (size_t)nTiles * 2 * T);
+    o_prz = carve(&off, sizeof(float4) * nTiles);
+    o_gpart = carve(&off, sizeof(float) * (size_t)nGroups * 2 * T);
+    o_grz = carve(&off, sizeof(float4) * nGroups);
+    o_cnt = carve(&off, sizeof(unsigned) * 2 * (nGroups + 1));
+    o_costs = d_costs ? 0 : carve(&off, sizeof(double) * K);
+    o_coll = carve(&off, (size_t)K);
+    o_Ustar = carve(&off, sizeof(double) * 2 * T);
+    if (off <= kStaticScratchBytes) break;
+  }
+  if (off > kStaticScratchBytes)
+    return fail(MPPI_EINVAL, "step needs %zu bytes of static scratch, the limit is %zu", off,
+                kStaticScratchBytes);
   StepFn fn = nullptr;  // picked before anything is launched
   rc = choose_step_kernel(p->model, c.tl.positions_per_thread, c.tl.threads, c.smem, nTiles,
                           p->sgf_window > 0 ? kFormSgf : kFormPlain, &fn);
   if (rc) return rc;
-  size_t off = 0;
-  const size_t o_st = carve(&off, sizeof(DevState));
-  const size_t o_cU = carve(&off, sizeof(float2) * T);
-  const size_t o_cA = carve(&off, sizeof(float2) * T);
-  const size_t o_cw = carve(&off, cw_bytes(p));
-  const size_t o_obst = carve(&off, (size_t)align_up(24 * (J > 0 ? J : 1), 16));
-  const size_t o_part = carve(&off, sizeof(float) * (size_t)nTiles * 2 * T);
-  const size_t o_prz = carve(&off, sizeof(float4) * nTiles);
-  const size_t o_gpart = carve(&off, sizeof(float) * (size_t)nGroups * 2 * T);
-  const size_t o_grz = carve(&off, sizeof(float4) * nGroups);
-  const size_t o_cnt = carve(&off, sizeof(unsigned) * 2 * (nGroups + 1));
-  const size_t o_costs = d_costs ? 0 : carve(&off, sizeof(double) * K);
-  const size_t o_coll = carve(&off, (size_t)K);
-  const size_t o_Ustar = carve(&off, sizeof(double) * 2 * T);
-  if (off > kStaticScratchBytes)
-    return fail(MPPI_EINVAL, "step needs %zu bytes of static scratch, the limit is %zu", off,
-                kStaticScratchBytes);
   cudaStream_t s = (cudaStream_t)stream;
   c.d_U = d_U;
   c.d_cU = (float2*)(base + o_cU);
