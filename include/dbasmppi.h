@@ -191,14 +191,14 @@ int mppi_step_device(mppi_ctx* c, const double* d_x0, const double* d_xref,
  * the plant after the update (first element of U* of Eq. 4), and, if U is
  * not NULL, the shifted nominal sequence for the next step (T x 2;
  * Algorithm 1's receding-horizon shift, the last element repeated).
- * After mppi_step, u0 and the status word are written by the step itself
- * into mapped pinned host memory, followed (after a system-scope fence) by
- * the step's iteration number.  With U NULL the call then returns as soon
+ * After mppi_step, u0, the status word and the sequence are written by the
+ * step itself into mapped pinned host memory, followed (after a system-scope
+ * fence) by the step's iteration number.  The call then returns as soon
  * as that number shows the last enqueued step, which can be before its
  * kernel has retired; the stream keeps the order of later work.  If the
- * stream ends without it (an error), when U is asked for, or after
- * mppi_step_device, it synchronises with the context's last stream and
- * copies what the mirror does not hold.  Errors: MPPI_ESTATE (no step has run),
+ * stream ends without it (an error), when U is asked for after
+ * mppi_set_state, or after mppi_step_device, it synchronises with the
+ * context's last stream and copies what the mirror does not hold.  Errors: MPPI_ESTATE (no step has run),
  * MPPI_ETIMEOUT (a bounded device wait of the step expired), MPPI_ECUDA. */
 int mppi_get_control(mppi_ctx* c, double* u0, double* U);
 
@@ -212,7 +212,7 @@ int mppi_get_debug(mppi_ctx* c, double* costs, uint8_t* collided,
 
 /* Bytes one mppi_step() moves host -> device (x0 and xref, read by the
  * kernel from the mapped staging) and device -> host for one
- * mppi_get_control(c, u0, NULL) (u0 and the status word, written by the
+ * mppi_get_control() (u0, the status word and the sequence, written by the
  * step into the mapped mirror). */
 int mppi_io_bytes(mppi_ctx* c, uint64_t* h2d, uint64_t* d2h);
 

@@ -222,17 +222,26 @@ int num_sms() {
 }
 
 // Largest dynamic shared memory a step kernel may request: the opt-in
-// per-block maximum less the kernel's static shared memory.
+// per-block maximum less the kernel's static shared memory.  Asked once per
+// device: the allocation-free entry point comes here on every step.
+constexpr int kMaxPickDevices = 64;
 int max_smem_optin() {
+  static std::atomic<int> memo[kMaxPickDevices];
   int dev = 0, v = 0;
   cudaGetDevice(&dev);
+  const bool in = dev >= 0 && dev < kMaxPickDevices;
+  if (in && (v = memo[dev].load(std::memory_order_relaxed)) > 0) return v;
   cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (v <= 0) v = 48 * 1024;
+  const bool known = v > 0;
+  if (!known) v = 48 * 1024;
   cudaFuncAttributes fa;
   size_t stat = 0;
-  if (cudaFuncGetAttributes(&fa, step_q14) == cudaSuccess) stat = fa.sharedSizeBytes;
+  const bool asked = cudaFuncGetAttributes(&fa, step_q14) == cudaSuccess;
+  if (asked) stat = fa.sharedSizeBytes;
   else cudaGetLastError();
-  return v - (int)align_up((int)stat + 64, 128);
+  v -= (int)align_up((int)stat + 64, 128);
+  if (in && known && asked) memo[dev].store(v, std::memory_order_relaxed);
+  return v;
 }
 
 // Step kernel of a launch: the 96-register form, or the 80-register form
@@ -241,7 +250,6 @@ int max_smem_optin() {
 // of a model's step kernels is raised once per device; the last decision per
 // device is kept, so a repeated configuration costs no occupancy query
 // (the allocation-free entry point calls this every step).
-constexpr int kMaxPickDevices = 64;
 struct PickMemo {
   int model, npos, threads, smem, nTiles;
   StepFn fn;
@@ -337,16 +345,19 @@ struct mppi_ctx {
   int in_next = 0;
   DevState* h_st = nullptr; // pinned readback
   double* h_U = nullptr;    // pinned readback
-  HostOut* h_out = nullptr;      // mapped mirror of u0 and status, written by the step
+  HostOut* h_out = nullptr;      // mapped mirror of u0, status and the sequence, written by the step
   HostOut* h_out_dev = nullptr;  // its device alias
   cudaStream_t own = nullptr;
   cudaStream_t last = nullptr;
   bool stepped = false;
   bool mirrored = false;  // the last step writes the host mirror (mppi_step)
+  bool mirror_U = false;  // and the sequence has not been set from the host since
   uint64_t iter = 0;  // iteration counter of the device state after the steps enqueued so far
 };
 
 namespace {
+
+size_t host_out_bytes(int T) { return sizeof(HostOut) + 2 * sizeof(double) * (size_t)T; }
 
 // The form of step kernel a context needs: the grid map's when it has one,
 // else the smoothing form when it smooths, else the plain one.
@@ -633,13 +644,13 @@ int mppi_create_tiled(const mppi_params* p, const double* u_init, const mppi_til
       return fail(MPPI_ENOMEM, "mapped pinned host allocation failed");
     }
   }
-  if (cudaHostAlloc((void**)&c->h_out, sizeof(HostOut), cudaHostAllocMapped) != cudaSuccess ||
+  if (cudaHostAlloc((void**)&c->h_out, host_out_bytes(T), cudaHostAllocMapped) != cudaSuccess ||
       cudaHostGetDevicePointer((void**)&c->h_out_dev, c->h_out, 0) != cudaSuccess) {
     cudaGetLastError();
     free_ctx(c);
     return fail(MPPI_ENOMEM, "mapped pinned host allocation failed");
   }
-  memset(c->h_out, 0, sizeof(HostOut));
+  memset(c->h_out, 0, host_out_bytes(T));
   if (cudaMallocHost((void**)&c->h_st, sizeof(DevState)) != cudaSuccess ||
       cudaMallocHost((void**)&c->h_U, sizeof(double) * 2 * T) != cudaSuccess) {
     cudaGetLastError();
@@ -811,7 +822,7 @@ int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream,
   CK(cudaGetLastError());
   c->last = s;
   c->stepped = true;
-  c->mirrored = mirror;
+  c->mirrored = c->mirror_U = mirror;
   ++c->iter;
   return MPPI_OK;
 }
@@ -850,10 +861,10 @@ int mppi_step(mppi_ctx* c, const double* x0, const double* xref, void* stream) {
 int mppi_get_control(mppi_ctx* c, double* u0, double* U) {
   if (!c) return fail(MPPI_ESTATE, "context is NULL");
   if (!c->stepped) return fail(MPPI_ESTATE, "no step has run");
-  // u0 and the status word come from the mapped mirror the step's final
-  // stage wrote; only U, when asked for, is copied
-  if (!U && c->mirrored) {
-    // the last step's final stage stores seq after its u0 and status (and a
+  // u0, the status word and the sequence come from the mapped mirror the
+  // step's final stage wrote
+  if (c->mirrored && (!U || c->mirror_U)) {
+    // the last step's final stage stores seq after its outputs (and a
     // system-scope fence): once seq shows that step, the mirror holds its
     // output, without waiting for the kernel to retire.  The stream is
     // polled now and then, so a step that ended without writing (an error)
@@ -870,6 +881,7 @@ int mppi_get_control(mppi_ctx* c, double* u0, double* U) {
           u0[0] = o->u0[0];
           u0[1] = o->u0[1];
         }
+        if (U) memcpy(U, c->h_out + 1, sizeof(double) * 2 * c->p.T);
         return MPPI_OK;
       }
       if ((n & 1023u) == 0u && cudaStreamQuery(c->last) != cudaErrorNotReady) break;
@@ -925,7 +937,7 @@ int mppi_get_debug(mppi_ctx* c, double* costs, uint8_t* collided, double* weight
 int mppi_io_bytes(mppi_ctx* c, uint64_t* h2d, uint64_t* d2h) {
   if (!c) return fail(MPPI_ESTATE, "context is NULL");
   if (h2d) *h2d = sizeof(double) * (uint64_t)(c->n + (c->p.T + 1) * c->n);
-  if (d2h) *d2h = sizeof(HostOut);  // u0 and the status word, written by the step
+  if (d2h) *d2h = host_out_bytes(c->p.T);  // the mirror, written by the step
   return MPPI_OK;
 }
 
@@ -972,6 +984,8 @@ int mppi_set_state(mppi_ctx* c, const double* U, double S_e, double beta, int32_
   st.iter = iter;
   st.status = 0;
   c->iter = iter;
+  c->mirror_U = false;
+  c->h_out->seq = (int)(uint32_t)iter;  // not the next step's number, wherever the count was before
   CK(cudaMemcpy(c->d_U, U, sizeof(double) * 2 * c->p.T, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(c->d_st, &st, sizeof(DevState), cudaMemcpyHostToDevice));
   prep_kernel<<<1, 256, 0, c->own>>>(c->D, 0);

@@ -498,6 +498,7 @@ __device__ __forceinline__ void final_stage(const CtrlDesc& D, char* smem, const
       D.Ustar[c] = us[d];
       D.U[c] = un[d];
     }
+    if (D.host_out) reinterpret_cast<double2*>(D.host_out + 1)[t] = make_double2(un[0], un[1]);
     if (t == 0) {
       us0[0] = us[0];
       us0[1] = us[1];
