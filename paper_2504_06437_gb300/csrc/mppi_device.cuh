@@ -745,6 +745,11 @@ __device__ __forceinline__ void far_eval(const FarCell* __restrict__ cell, const
   }
 }
 
+template <bool B>
+struct BoolC {
+  static constexpr bool value = B;
+};
+
 // Fused barrier over nunits = T S (step, sample) units; unit u = t S + s has
 // its pose at pose[t SP + s] (SP = row_stride(S, BATCHED)) and P shape
 // points shp[0..P).  A warp takes groups of 32 (NPOS / P) consecutive units
@@ -822,8 +827,8 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
     // obstacles in pairs: 1/h1 + 1/h2 = (h1 + h2) / (h1 h2), one reciprocal
     // for two terms (h1 h2 stays finite for |p - c| < 4e9 m and h_eps >= 1e-18);
     // with more points per thread the pair's temporaries would not fit
-    auto two = [&](const float4 o, const float4 q) {
-      if constexpr (NPOS <= 8) {
+    auto two = [&](const float4 o, const float4 q, auto paired) {
+      if constexpr (decltype(paired)::value) {
         const float2 nox = make_float2(-o.x, -o.x), noy = make_float2(-o.y, -o.y);
         const float2 noz = make_float2(o.z, o.z);
         const float2 nqx = make_float2(-q.x, -q.x), nqy = make_float2(-q.y, -q.y);
@@ -855,12 +860,12 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
       int j = 0;
       for (; j + 1 < nn; j += 2) {
         const unsigned jj = *reinterpret_cast<const unsigned*>(l + j);
-        two(obs4[jj & 0xffffu], obs4[jj >> 16]);
+        two(obs4[jj & 0xffffu], obs4[jj >> 16], BoolC<true>());
       }
       if (j < nn) one(obs4[l[j]]);
     } else {
       int j = 0;
-      for (; j + 1 < J; j += 2) two(obs4[j], obs4[j + 1]);
+      for (; j + 1 < J; j += 2) two(obs4[j], obs4[j + 1], BoolC<(NPOS <= 8)>());
       if (j < J) one(obs4[j]);
     }
     if constexpr (GRID) {
