@@ -248,7 +248,8 @@ int mppi_autotune_flush(const mppi_params* p, const double* cxcyr, int32_t J, co
                         int32_t nx, int32_t ny, double ox, double oy, double res, int32_t iters,
                         uint64_t flush_bytes, mppi_tiling* best, float* best_us);
 
-/* The launch shape in use and the number of CTAs of one step. */
+/* The launch shape in use and the number of tiles (of samples_per_cta samples)
+ * of one step; in grids of many waves a CTA takes several of them in a row. */
 int mppi_get_tiling(mppi_ctx* c, mppi_tiling* t, int32_t* n_ctas);
 
 /* Register cap of the step kernel the context launches: 96, or 80 when the

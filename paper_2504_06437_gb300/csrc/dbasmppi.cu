@@ -201,12 +201,27 @@ size_t cw_bytes(const mppi_params* p) {
   return sizeof(float) * ((size_t)sgf_table_offset(p->T) + (size_t)p->sgf_window * p->sgf_window);
 }
 
+// Tiles that one CTA takes in a row (the prologue once): 1, 2, 4 or 8.
+constexpr int kMaxChunk = 8;
+
 // Tiles merged by one CTA: all of them in one level up to 256 tiles, else
-// groups of at least 32 so that at most 64 group results remain.
+// groups of at least 32, of whole chunks of tiles, so that at most 64 group
+// results remain.
 int group_size(int nTiles) {
   if (nTiles <= 256) return nTiles;
-  int GT = (nTiles + 63) / 64;
+  int GT = ((nTiles + 63) / 64 + kMaxChunk - 1) / kMaxChunk * kMaxChunk;
   return GT < 32 ? 32 : GT;
+}
+
+// Chunk of a grid that finds room for `resident` CTAs at a time: at least
+// three waves of chunks, since the last wave of larger ones leaves more of the
+// GPU idle than the prologues cost.  Unicycle K 65536 (7 waves of tiles)
+// 311 us tile by tile, 305 in twos, 324 in fours; quadrotor K 32768 (3.5
+// waves) 753 tile by tile, 825 in twos.
+int chunk_of(long nTiles, long resident) {
+  int c = 1;
+  while (c < kMaxChunk && nTiles >= 6 * c * resident) c *= 2;
+  return c;
 }
 
 int g_num_sms = 0;
@@ -251,7 +266,7 @@ int max_smem_optin() {
 // device is kept, so a repeated configuration costs no occupancy query
 // (the allocation-free entry point calls this every step).
 struct PickMemo {
-  int model, npos, threads, smem, nTiles;
+  int model, npos, threads, smem, nTiles, chunk;
   StepFn fn;
 };
 std::mutex g_pick_mu;
@@ -260,7 +275,7 @@ bool g_form_attr[kMaxPickDevices][2][MPPI_NUM_MODELS] = {};
 PickMemo g_pick_memo[kMaxPickDevices] = {};
 
 int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, int form,
-                       StepFn* out) {
+                       StepFn* out, int* chunk) {
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxPickDevices) return fail(MPPI_EINVAL, "device %d out of range", dev);
@@ -275,6 +290,9 @@ int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, i
       done = true;
     }
     *out = pick_form_kernel(form, model, npos);
+    int occ = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, *out, threads, smem));
+    *chunk = chunk_of(nTiles, (long)std::max(occ, 1) * num_sms());
     return MPPI_OK;
   }
   // only this model's kernels: with lazy module loading, touching a kernel
@@ -291,6 +309,7 @@ int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, i
   if (m.fn && m.model == model && m.npos == npos && m.threads == threads && m.smem == smem &&
       m.nTiles == nTiles) {
     *out = m.fn;
+    *chunk = m.chunk;
     return MPPI_OK;
   }
   const StepFn hi = pick_kernel(model, npos, false), lo = pick_kernel(model, npos, true);
@@ -298,7 +317,8 @@ int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, i
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_hi, hi, threads, smem));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_lo, lo, threads, smem));
   const StepFn fn = (occ_lo > occ_hi && (long)nTiles > (long)occ_hi * num_sms()) ? lo : hi;
-  m = PickMemo{model, npos, threads, smem, nTiles, fn};
+  *chunk = chunk_of(nTiles, (long)std::max(fn == lo ? occ_lo : occ_hi, 1) * num_sms());
+  m = PickMemo{model, npos, threads, smem, nTiles, *chunk, fn};
   *out = fn;
   return MPPI_OK;
 }
@@ -504,6 +524,7 @@ void fill_desc(mppi_ctx* c) {
   D.S = c->tl.samples_per_cta;
   D.NPOS = c->tl.positions_per_thread;
   D.nc = c->nc;
+  D.chunk = 1;
   D.nTiles = (p->K + D.S - 1) / D.S;
   D.GT = group_size(D.nTiles);
   D.nGroups = (D.nTiles + D.GT - 1) / D.GT;
@@ -666,8 +687,7 @@ int mppi_create_tiled(const mppi_params* p, const double* u_init, const mppi_til
   c->last = c->own;
   fill_desc(c);
   rc = choose_step_kernel(p->model, c->tl.positions_per_thread, c->tl.threads, c->smem, nTiles,
-                          p->sgf_window > 0 ? kFormSgf : kFormPlain,
-                          &c->fn);
+                          p->sgf_window > 0 ? kFormSgf : kFormPlain, &c->fn, &c->D.chunk);
   if (rc) {
     free_ctx(c);
     return rc;
@@ -729,8 +749,9 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   if (t.samples_per_cta != c->tl.samples_per_cta)
     return fail(MPPI_EINVAL, "obstacle set too large for the controller's tile shape");
   StepFn fn = nullptr;
+  int chunk = 1;
   rc = choose_step_kernel(c->p.model, t.positions_per_thread, t.threads, smem, c->D.nTiles,
-                          step_form(c), &fn);
+                          step_form(c), &fn, &chunk);
   if (rc) return rc;
   c->tl = t;
   c->smem = smem;
@@ -738,6 +759,7 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   c->fn = fn;
   c->D.J = J;
   c->D.nc = nc;
+  c->D.chunk = chunk;
   c->D.obst = c->d_obst;
   return MPPI_OK;
 }
@@ -765,9 +787,11 @@ int mppi_set_grid(mppi_ctx* c, const float* sdf, int32_t nx, int32_t ny, double 
     if (int rc = check_grid(sdf, nx, ny, ox, oy, res)) return rc;
   }
   StepFn fn = nullptr;
+  int chunk = 1;
   int rc = choose_step_kernel(c->p.model, c->tl.positions_per_thread, c->tl.threads, c->smem,
                               c->D.nTiles,
-                              off ? (c->p.sgf_window > 0 ? kFormSgf : kFormPlain) : kFormGrid, &fn);
+                              off ? (c->p.sgf_window > 0 ? kFormSgf : kFormPlain) : kFormGrid, &fn,
+                              &chunk);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->last));  // no step in flight reads the old map
   float* nb = nullptr;
@@ -801,6 +825,7 @@ int mppi_set_grid(mppi_ctx* c, const float* sdf, int32_t nx, int32_t ny, double 
   cudaFree(c->d_grid);
   c->d_grid = nb;
   c->fn = fn;
+  c->D.chunk = chunk;
   return MPPI_OK;
 }
 
@@ -813,11 +838,11 @@ namespace {
 int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream, bool mirror) {
   cudaStream_t s = stream ? (cudaStream_t)stream : c->own;
   if (mirror) {
-    c->fn<<<c->D.nTiles, c->tl.threads, c->smem, s>>>(c->D, x0, xref);
+    c->fn<<<(c->D.nTiles + c->D.chunk - 1) / c->D.chunk, c->tl.threads, c->smem, s>>>(c->D, x0, xref);
   } else {
     CtrlDesc D = c->D;
     D.host_out = nullptr;
-    c->fn<<<c->D.nTiles, c->tl.threads, c->smem, s>>>(D, x0, xref);
+    c->fn<<<(c->D.nTiles + c->D.chunk - 1) / c->D.chunk, c->tl.threads, c->smem, s>>>(D, x0, xref);
   }
   CK(cudaGetLastError());
   c->last = s;
@@ -1166,8 +1191,9 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
     return fail(MPPI_EINVAL, "step needs %zu bytes of static scratch, the limit is %zu", off,
                 kStaticScratchBytes);
   StepFn fn = nullptr;  // picked before anything is launched
+  int chunk = 1;
   rc = choose_step_kernel(p->model, c.tl.positions_per_thread, c.tl.threads, c.smem, nTiles,
-                          p->sgf_window > 0 ? kFormSgf : kFormPlain, &fn);
+                          p->sgf_window > 0 ? kFormSgf : kFormPlain, &fn, &chunk);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   c.d_U = d_U;
@@ -1187,11 +1213,12 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   c.d_Ustar = (double*)(base + o_Ustar);
   fill_desc(&c);
   c.D.J = J;
+  c.D.chunk = chunk;
   if (J > 0)
     CK(cudaMemcpyAsync(c.d_obst, d_obst, sizeof(double) * 3 * J, cudaMemcpyDeviceToDevice, s));
   static_prologue<<<1, 256, 0, s>>>(c.D, d_ctl, 2 * (nGroups + 1));
   CK(cudaGetLastError());
-  fn<<<c.D.nTiles, c.tl.threads, c.smem, s>>>(c.D, d_x0, d_xref);
+  fn<<<(nTiles + chunk - 1) / chunk, c.tl.threads, c.smem, s>>>(c.D, d_x0, d_xref);
   CK(cudaGetLastError());
   static_epilogue<<<1, 32, 0, s>>>(c.d_st, d_ctl, d_u0);
   CK(cudaGetLastError());
@@ -1767,6 +1794,22 @@ int lane_step(mppi_batch* b, BatchLane& L, const int32_t* slots, int32_t n, cons
     smem = std::max(smem, s.smem);
     order[i] = i;
   }
+  // batch_kernel covers the unicycle and the 6-state quadrotor; a step that
+  // holds the Ackermann vehicle or the 5-state quadrotor takes batch_kernel_all
+  bool all_models = false;
+  for (int i = 0; i < n; ++i) all_models = all_models || b->slots[slots[i]].p.model >= 2;
+  const auto kernel = all_models ? batch_kernel_all : batch_kernel;
+  int occ = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kBatchThreads, smem));
+  if (occ < 1) return fail(MPPI_EINVAL, "batch needs %d bytes of shared memory per CTA", smem);
+  // tiles that share a work item (and its prologue): enough items are left
+  // for every resident CTA to take twelve or more, so that the last ones even
+  // out (512 controllers 14.2 ms tile by tile, 13.1 ms in fours)
+  const int chunk = std::min(4, chunk_of((long)n_items / 4, (long)num_sms() * occ));
+  if (chunk > 1) {
+    n_items = 0;
+    for (int i = 0; i < n; ++i) n_items += (b->slots[slots[i]].D.nTiles + chunk - 1) / chunk;
+  }
   const size_t head = sizeof(BatchHdr) + sizeof(StepEntry) * n + sizeof(WorkItem) * n_items;
   const size_t inputs_off = (head + 15) & ~(size_t)15;
   const size_t bytes = inputs_off + sizeof(double) * n_in;
@@ -1801,20 +1844,13 @@ int lane_step(mppi_batch* b, BatchLane& L, const int32_t* slots, int32_t n, cons
   for (int oi = 0; oi < n; ++oi) {
     const int i = order[oi];
     const BatchSlot& s = b->slots[slots[i]];
-    for (int t = 0; t < s.D.nTiles; ++t) items[w++] = WorkItem{i, t};
+    for (int t = 0; t < s.D.nTiles; t += chunk) items[w++] = WorkItem{i, t};
   }
   hdr->n_steps = n;
   hdr->n_items = (int)n_items;
   hdr->next = 0u;
   hdr->inputs_off = (int)inputs_off;
-  // batch_kernel covers the unicycle and the 6-state quadrotor; a step that
-  // holds the Ackermann vehicle or the 5-state quadrotor takes batch_kernel_all
-  bool all_models = false;
-  for (int i = 0; i < n; ++i) all_models = all_models || b->slots[slots[i]].p.model >= 2;
-  const auto kernel = all_models ? batch_kernel_all : batch_kernel;
-  int occ = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kBatchThreads, smem));
-  if (occ < 1) return fail(MPPI_EINVAL, "batch needs %d bytes of shared memory per CTA", smem);
+  hdr->chunk = chunk;
   int grid = (int)std::min<size_t>((size_t)num_sms() * occ, n_items);
   if (share < 1.0) grid = std::max(1, std::min(grid, (int)(share * num_sms() * occ)));
   std::vector<int> key(slots, slots + n);
@@ -2268,6 +2304,12 @@ int ring_alloc(mppi_server* sv) {
   return MPPI_OK;
 }
 
+// Tiles of one item of the device queue.  A CTA reads an item, its request
+// and the request's inputs from host memory, some microseconds over the host
+// link, before it runs the tiles; a large request has items to spare for
+// every CTA, a small one is spread as far as it goes.
+int serve_chunk(int nTiles) { return nTiles >= 512 ? 4 : nTiles >= 256 ? 2 : 1; }
+
 // One pass of the device-queue scheduler: completions, publication of
 // queued requests, and a launch of the resident kernel when work is
 // published and none runs.  Returns whether anything happened.
@@ -2342,7 +2384,8 @@ bool ring_step(mppi_server* sv, bool dev_ok) {
       ServerReq& r = qu.front();
       if (cap > 0 && R.flight_ops[c] > 0 && R.flight_ops[c] + r.ops > cap) break;
       const BatchSlot& s = sv->b->slots[r.robot];
-      const unsigned nt = (unsigned)s.D.nTiles;
+      const int chunk = serve_chunk(s.D.nTiles);
+      const unsigned nt = (unsigned)((s.D.nTiles + chunk - 1) / chunk);
       if (s.smem > R.max_dyn) {  // cannot run in the serving kernel at all
         ServerDone d;
         d.robot = r.robot;
@@ -2376,10 +2419,10 @@ bool ring_step(mppi_server* sv, bool dev_ok) {
       } else {
         for (int t = 0; t <= T; ++t) memcpy(in + n + (size_t)t * n, s.p.x_goal, sizeof(double) * n);
       }
-      R.h_reqs[rq] = ServeReq{r.robot, n, n * (T + 2), R.seq};
+      R.h_reqs[rq] = ServeReq{r.robot, n, n * (T + 2), R.seq, chunk, 0};
       WorkItem* items = R.h_items[c];
       for (unsigned t = 0; t < nt; ++t)
-        items[(R.pub[c] + t) & (R.cap_items - 1u)] = WorkItem{rq, (int)t};
+        items[(R.pub[c] + t) & (R.cap_items - 1u)] = WorkItem{rq, (int)t * chunk};
       RingReq x;
       x.r = std::move(r);
       x.rq = rq;

@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel_all(
   if (tid == 0) mbar_init(&ts.mbar);
   __syncthreads();
   uint32_t phase = 0u;
-  const int n_items = hdr->n_items;
+  const int n_items = hdr->n_items, chunk = hdr->chunk;
   for (;;) {
     if (tid == 0) s_item = (int)atomicAdd(&hdr->next, 1u);
     __syncthreads();
@@ -41,14 +41,14 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel_all(
     double* uo = u0_out + 8 * w.ctrl;  // u0 and the predicted next state
     // the batched form of the tile: see run_tile
     switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-      case 0: run_tile<0, 8>(w.tile, x0, xref, phase, uo); break;
-      case 1: run_tile<0, 14>(w.tile, x0, xref, phase, uo); break;
-      case 2: run_tile<1, 8>(w.tile, x0, xref, phase, uo); break;
-      case 3: run_tile<1, 14>(w.tile, x0, xref, phase, uo); break;
-      case 4: run_tile<2, 8>(w.tile, x0, xref, phase, uo); break;
-      case 5: run_tile<2, 14>(w.tile, x0, xref, phase, uo); break;
-      case 6: run_tile<3, 8>(w.tile, x0, xref, phase, uo); break;
-      default: run_tile<3, 14>(w.tile, x0, xref, phase, uo); break;
+      case 0: run_tile<0, 8>(w.tile, chunk, x0, xref, phase, uo); break;
+      case 1: run_tile<0, 14>(w.tile, chunk, x0, xref, phase, uo); break;
+      case 2: run_tile<1, 8>(w.tile, chunk, x0, xref, phase, uo); break;
+      case 3: run_tile<1, 14>(w.tile, chunk, x0, xref, phase, uo); break;
+      case 4: run_tile<2, 8>(w.tile, chunk, x0, xref, phase, uo); break;
+      case 5: run_tile<2, 14>(w.tile, chunk, x0, xref, phase, uo); break;
+      case 6: run_tile<3, 8>(w.tile, chunk, x0, xref, phase, uo); break;
+      default: run_tile<3, 14>(w.tile, chunk, x0, xref, phase, uo); break;
     }
     __syncthreads();  // Ds and s_item are reused by the next item
   }

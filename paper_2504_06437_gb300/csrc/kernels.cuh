@@ -100,7 +100,7 @@ __global__ void step_p8_grid(const __grid_constant__ CtrlDesc D, const double* _
 __global__ void step_p14_grid(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,
                               const double* __restrict__ xref);
 
-// Batched step: persistent CTAs pull (controller, tile) work items.
+// Batched step: persistent CTAs pull (controller, first tile) work items.
 struct WorkItem {
   int ctrl;  // index into the step table
   int tile;
@@ -115,6 +115,7 @@ struct BatchHdr {
   int n_steps, n_items;
   unsigned next;
   int inputs_off;  // byte offset of the packed inputs
+  int chunk, pad[3];  // tiles of a work item (from its tile on, within the controller)
 };
 constexpr int kBatchThreads = 256;
 __global__ void batch_kernel(const CtrlDesc* __restrict__ descs, unsigned char* stage,
@@ -141,12 +142,14 @@ struct __align__(8) ServeHdr {
   unsigned pad;
 };
 // One published request: the robot's pool slot, where its reference starts
-// in its inputs, how many input doubles there are, and its sequence number.
+// in its inputs, how many input doubles there are, its sequence number and
+// the tiles of its items.
 struct ServeReq {
   int slot;
   int xref_off;
   int n_in;
   unsigned seq;
+  int chunk, pad;  // tiles of an item, from its tile on
 };
 struct ServeRing {
   const ServeHdr* hdr;          // mapped host memory (device alias)
@@ -232,6 +235,7 @@ __device__ __forceinline__ void serve_body(const CtrlDesc* __restrict__ descs, c
     const int xref_off = *reinterpret_cast<const volatile int*>(&ep->xref_off);
     const int n_in = *reinterpret_cast<const volatile int*>(&ep->n_in);
     const unsigned seq = *reinterpret_cast<const volatile unsigned*>(&ep->seq);
+    const int chunk = *reinterpret_cast<const volatile int*>(&ep->chunk);
     const int* src = reinterpret_cast<const int*>(descs + slot);
     int* dst = reinterpret_cast<int*>(&Ds);
     for (int i = tid; i < (int)(sizeof(CtrlDesc) / 4); i += blockDim.x) dst[i] = __ldcg(src + i);
@@ -242,17 +246,17 @@ __device__ __forceinline__ void serve_body(const CtrlDesc* __restrict__ descs, c
     const double* x0 = s_in;
     const double* xref = s_in + xref_off;
     switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-      case 0: run_tile<0, 8>(tile, x0, xref, phase, uo); break;
-      case 1: run_tile<0, 14>(tile, x0, xref, phase, uo); break;
-      case 2: run_tile<1, 8>(tile, x0, xref, phase, uo); break;
-      case 3: run_tile<1, 14>(tile, x0, xref, phase, uo); break;
+      case 0: run_tile<0, 8>(tile, chunk, x0, xref, phase, uo); break;
+      case 1: run_tile<0, 14>(tile, chunk, x0, xref, phase, uo); break;
+      case 2: run_tile<1, 8>(tile, chunk, x0, xref, phase, uo); break;
+      case 3: run_tile<1, 14>(tile, chunk, x0, xref, phase, uo); break;
       default:
         if constexpr (ALL) {
           switch (Ds.model * 2 + npos_code(Ds.NPOS)) {
-            case 4: run_tile<2, 8>(tile, x0, xref, phase, uo); break;
-            case 5: run_tile<2, 14>(tile, x0, xref, phase, uo); break;
-            case 6: run_tile<3, 8>(tile, x0, xref, phase, uo); break;
-            default: run_tile<3, 14>(tile, x0, xref, phase, uo); break;
+            case 4: run_tile<2, 8>(tile, chunk, x0, xref, phase, uo); break;
+            case 5: run_tile<2, 14>(tile, chunk, x0, xref, phase, uo); break;
+            case 6: run_tile<3, 8>(tile, chunk, x0, xref, phase, uo); break;
+            default: run_tile<3, 14>(tile, chunk, x0, xref, phase, uo); break;
           }
         }
         break;
@@ -275,7 +279,7 @@ __device__ __forceinline__ void step_body(const CtrlDesc& D, const double* __res
   if (threadIdx.x == 0) mbar_init(&ts.mbar);
   __syncthreads();
   uint32_t phase = 0u;
-  run_tile_inl<MODEL, NPOS, false, SGF, GRID>(D, blockIdx.x, x0, xref, phase);
+  run_tile_inl<MODEL, NPOS, false, SGF, GRID>(D, blockIdx.x * D.chunk, D.chunk, x0, xref, phase);
 }
 
 }  // namespace dbm

@@ -101,6 +101,7 @@ struct __align__(16) HostOut {
 struct CtrlDesc {
   int model, K, T, J, P, n;
   int S, NPOS, nTiles, GT, nGroups;
+  int chunk;                 // tiles of a CTA of the one-controller kernels
   int nc;                    // far-field cells of a tile (far_cells), 0 = every pair directly
   float r_body;              // largest distance of a shape point from the body's position
   float dt, h_eps, C_coll, ln_mu, ln_sigma;

@@ -738,7 +738,10 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   }
 }
 
-// One tile of one controller.  ts.mbar must be initialised; mbar_phase is
+// `count` tiles of one controller, from tile0 on and all of one merge group
+// (a multiple of count tiles): the prologue and the ticket once, the rest tile
+// by tile, each with its own row of partials, so the results do not depend
+// on how tiles are shared out.  ts.mbar must be initialised; mbar_phase is
 // each thread's own copy of the parity of the barrier's next completion.
 // BATCHED: the tile runs in the persistent batch kernel, which takes the
 // one-batch form of merge_partials and the odd row stride of row_stride;
@@ -755,7 +758,7 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
 // kernels call it out of line (run_tile), which keeps their four-model
 // switch small.
 template <int MODEL, int NPOS, bool BATCHED, bool SGF = BATCHED, bool GRID = false>
-__device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
+__device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int count,
                                              const double* __restrict__ x0g,
                                              const double* __restrict__ xrefg, uint32_t& mbar_phase,
                                              double* u0_out = nullptr) {
@@ -783,7 +786,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
   float* xi = reinterpret_cast<float*>(smem + L.xi);
   double* red = reinterpret_cast<double*>(smem + L.red);
   DevState* st = D.st;
-  const int k0 = tile * S;
+  const int t_end = min(tile0 + count, D.nTiles);  // this CTA's tiles: [tile0, t_end)
 
   // ---- prologue: stage obstacles (TMA bulk copy), per-step constants
   __syncthreads();  // previous use of shared memory by this CTA is over
@@ -900,6 +903,8 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
     }
   }
 
+  for (int tile = tile0;;) {  // (the body is not indented)
+  const int k0 = tile * S;
   // ---- noise: every (sample, step) draw, kept as the clamped control
   {
     const uint32_t it_lo = (uint32_t)(st->iter & 0xffffffffull);
@@ -928,7 +933,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
   }
   __syncthreads();
   // (one lane of the last warp, which has the fewest samples below)
-  if (tid == nthreads - 32) {
+  if (tid == nthreads - 32 && tile == tile0) {
     float fbd = 0.0f, fb0 = 0.0f;
     for (int w = 0; w < nwarps; ++w) {
       fbd += reinterpret_cast<const float*>(red)[2 * w];
@@ -1041,20 +1046,24 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
     }
   }
 
+  __syncthreads();
+  if (++tile == t_end) break;
+  }
+
   // ---- two-level last-arriver merge.  The CTA's writes are published by
   // one thread: barrier, fence, ticket; the last arriver fences again before
   // the barrier that releases its threads to read the others' partials.  The
   // merge reads (and clears) the group's minimum word, the exact minimum of
   // its members' rho.
-  __syncthreads();
-  const int g = tile / D.GT;
+  const int g = tile0 / D.GT;
   const int m0 = g * D.GT;
   const int members = min(D.GT, D.nTiles - m0);
   unsigned* minw = D.counters + D.nGroups + 1;
   if (tid == 0) {
     __threadfence();
-    unsigned tk = atomicAdd(&D.counters[g], 1u);
-    ts.flag = (tk == (unsigned)(members - 1));
+    const unsigned mine = (unsigned)(t_end - tile0);
+    unsigned tk = atomicAdd(&D.counters[g], mine);
+    ts.flag = (tk + mine == (unsigned)members);
     if (ts.flag) {
       __threadfence();
       D.counters[g] = 0u;
@@ -1094,7 +1103,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
                              nthreads);
   }
   // (one sample with all but 1 / kRefShare of the weight needs no second look)
-  if (nc > 0 && ts.Z.hi > 1.0f + 1.0f / kRefShare)
+  if (D.nc > 0 && ts.Z.hi > 1.0f + 1.0f / kRefShare)
     refine_samples<MODEL, NPOS, BATCHED, GRID>(D);
   if constexpr (SGF) {
     if (D.sgf_wp)
@@ -1112,10 +1121,10 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile,
 
 // The tile of the persistent kernels, whose descriptor is tile_desc().
 template <int MODEL, int NPOS>
-__device__ __noinline__ void run_tile(int tile, const double* __restrict__ x0g,
+__device__ __noinline__ void run_tile(int tile0, int count, const double* __restrict__ x0g,
                                       const double* __restrict__ xrefg, uint32_t& mbar_phase,
                                       double* u0_out) {
-  run_tile_inl<MODEL, NPOS, true>(tile_desc(), tile, x0g, xrefg, mbar_phase, u0_out);
+  run_tile_inl<MODEL, NPOS, true>(tile_desc(), tile0, count, x0g, xrefg, mbar_phase, u0_out);
 }
 
 }  // namespace dbm
