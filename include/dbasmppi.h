@@ -295,7 +295,9 @@ int mppi_debug_wait_probe(int64_t max_cycles, int32_t arrive);
  * The paper has no counterpart; it is the step of mppi_step_device() with its
  * scratch in a fixed 8 MiB array inside the library (each GPU that loads the
  * library keeps it until the process exits).
- *   d_obst   device, J x 3 (cx, cy, r); copied into the scratch.
+ *   d_obst   device, J x 3 (cx, cy, r); read by the enqueued work, like d_x0
+ *            and d_xref (an odd number, or one off a 16-byte boundary, is
+ *            copied into the scratch first).
  *   d_x0     device, n doubles;  d_xref device, (T+1) x n.
  *   d_U      device, T x 2, in/out: the nominal sequence; shifted on return.
  *   d_ctl    device, 5 doubles, in/out: {S_e, beta, first (1 before the

@@ -1092,9 +1092,11 @@ std::mutex g_static_mu;  // guards the set-up of g_static_base
 
 // Device-side copy of the caller's controller state into the scratch state
 // block, ticket counters and minimum words cleared, constants derived; the caller's ctl is
-// {S_e, beta, first, iter, status}.
+// {S_e, beta, first, iter, status}.  obst: the caller's obstacles, copied to
+// where the tiles' bulk copy can read them, or null where it reads them in
+// place.  The step's final stage writes the caller's state and control back.
 __global__ void static_prologue(const __grid_constant__ CtrlDesc D, const double* __restrict__ ctl,
-                                int n_counters) {
+                                const double* __restrict__ obst, int n_counters) {
   __shared__ double red[64];
   if (threadIdx.x == 0) {
     D.st->S_e = ctl[0];
@@ -1104,22 +1106,10 @@ __global__ void static_prologue(const __grid_constant__ CtrlDesc D, const double
     D.st->status = 0;
   }
   for (int i = threadIdx.x; i < n_counters; i += blockDim.x) D.counters[i] = 0u;
-  __syncthreads();
+  if (obst)
+    for (int i = threadIdx.x; i < 3 * D.J; i += blockDim.x) const_cast<double*>(D.obst)[i] = obst[i];
   init_constants(D, threadIdx.x, blockDim.x);
-  prep_constants(D, D.U, &D.st->S_e, red, threadIdx.x, blockDim.x);
-}
-
-__global__ void static_epilogue(const DevState* __restrict__ st, double* __restrict__ ctl,
-                                double* __restrict__ u0) {
-  if (threadIdx.x == 0) {
-    ctl[0] = st->S_e;
-    ctl[1] = st->beta;
-    ctl[2] = st->first;
-    ctl[3] = (double)st->iter;
-    ctl[4] = st->status;
-    u0[0] = st->u0[0];
-    u0[1] = st->u0[1];
-  }
+  prep_constants(D, D.U, ctl, red, threadIdx.x, blockDim.x);
 }
 
 size_t carve(size_t* off, size_t bytes) {
@@ -1214,13 +1204,16 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   fill_desc(&c);
   c.D.J = J;
   c.D.chunk = chunk;
-  if (J > 0)
-    CK(cudaMemcpyAsync(c.d_obst, d_obst, sizeof(double) * 3 * J, cudaMemcpyDeviceToDevice, s));
-  static_prologue<<<1, 256, 0, s>>>(c.D, d_ctl, 2 * (nGroups + 1));
+  c.D.ctl_out = d_ctl;
+  c.D.u0_out = d_u0;
+  // a tile's bulk copy takes whole 16-byte units from a 16-byte boundary: an
+  // even number of obstacles that starts on one is read where it lies
+  const bool in_place = J > 0 && J % 2 == 0 && ((uintptr_t)d_obst & 15u) == 0;
+  if (in_place) c.D.obst = d_obst;
+  static_prologue<<<1, 256, 0, s>>>(c.D, d_ctl, in_place || J == 0 ? nullptr : d_obst,
+                                    2 * (nGroups + 1));
   CK(cudaGetLastError());
   fn<<<(nTiles + chunk - 1) / chunk, c.tl.threads, c.smem, s>>>(c.D, d_x0, d_xref);
-  CK(cudaGetLastError());
-  static_epilogue<<<1, 32, 0, s>>>(c.d_st, d_ctl, d_u0);
   CK(cudaGetLastError());
   return MPPI_OK;
 }

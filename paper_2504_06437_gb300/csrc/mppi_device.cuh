@@ -137,6 +137,8 @@ struct CtrlDesc {
   uint8_t* coll;             // K
   double* Ustar;             // T x 2
   HostOut* host_out;         // device alias of the host mirror, or null
+  double* ctl_out;           // the allocation-free step: where the caller keeps its state
+  double* u0_out;            // and its control; null elsewhere
 };
 
 // The Savitzky-Golay weights (W x W floats, row q: the fit's value at window

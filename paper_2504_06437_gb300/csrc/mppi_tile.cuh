@@ -52,21 +52,33 @@ __device__ inline void sgf_weights(float* w, int W, int p, int tid, int nthreads
   }
 }
 
+// g^e for 0 <= e <= MPPI_MAX_T by repeated squaring: nine products in a row at
+// most, where pow takes several times as many FP64 operations; within e
+// roundings, far below the FP32 weights it goes into.
+__device__ __forceinline__ double pow_int(double g, int e) {
+  double r = 1.0;
+  for (; e; e >>= 1) {
+    if (e & 1) r *= g;
+    g *= g;
+  }
+  return r;
+}
+
 // Constants of the controller that never change: the unrolled DBaS weights
 // c_s (scaled by R_B) and their sums, and the smoothing weights.  One CTA, at
 // creation (and on every call of the allocation-free entry point).
 __device__ inline void init_constants(const CtrlDesc& D, int tid, int nthreads) {
   const int T = D.T;
   const double g = D.gamma_bas;
+  const double q = 1.0 / (1.0 - g);
   for (int t = tid; t < T; t += nthreads) {
     // step t produces x_{t+1}: c_{t+1} = (1 - g^(T - t)) / (1 - g)
-    double c = (1.0 - pow(g, (double)(T - t))) / (1.0 - g);
-    D.cw[t] = (float)(D.R_B_d * c);
+    D.cw[t] = (float)(D.R_B_d * ((1.0 - pow_int(g, T - t)) * q));
   }
-  if (tid == 0) {
-    double gT = pow(g, (double)T);
-    D.st->g1 = g * (1.0 - gT) / (1.0 - g);
-    D.st->csum = (T - D.st->g1) / (1.0 - g);
+  if (tid == nthreads - 1) {
+    const double g1 = g * (1.0 - pow_int(g, T)) * q;
+    D.st->g1 = g1;
+    D.st->csum = (T - g1) * q;
   }
   if (D.sgf_wp)
     sgf_weights(D.cw + sgf_table_offset(T), D.sgf_wp & 0xff, D.sgf_wp >> 8, tid, nthreads);
@@ -570,6 +582,15 @@ __device__ __forceinline__ void final_stage(const CtrlDesc& D, char* smem, const
       xn[1] = ts.x0[1] + (double)x1[1];
       for (int d = 2; d < n; ++d) xn[d] = (double)x1[d];
       for (int d = 0; d < 6; ++d) st->x1[d] = xn[d];
+      if (D.ctl_out) {  // the allocation-free step: the caller's state and control
+        D.ctl_out[0] = S_e_next;
+        D.ctl_out[1] = ts.beta0;
+        D.ctl_out[2] = 0.0;
+        D.ctl_out[3] = (double)(ts.iter + 1ull);
+        D.ctl_out[4] = (double)*reinterpret_cast<volatile int*>(&st->status);
+        D.u0_out[0] = us0[0];
+        D.u0_out[1] = us0[1];
+      }
       if (out) {  // batched launches: u0 then the predicted state, 8 doubles
         out[0] = us0[0];
         out[1] = us0[1];
