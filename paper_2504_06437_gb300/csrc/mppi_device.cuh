@@ -324,9 +324,15 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
   return c;
 }
 
-// Top 23 bits of r as an odd multiple of 2^-24: exactly representable.
+// The top 23 bits k of r as an odd multiple (2 k + 1) of 2^-24, times `scale`
+// (1 or 2): exactly representable, so 1 + k 2^-23, whose bits are put
+// together, less 1 - 2^-24 is exact (no integer conversion, which runs at a
+// quarter of the rate).
+template <int SCALE>
 __device__ __forceinline__ float unit_open(uint32_t r) {
-  return __uint2float_rn((r >> 8) | 1u) * 5.9604644775390625e-8f;
+  static_assert(SCALE == 1 || SCALE == 2, "one exponent up at most");
+  const uint32_t one = SCALE == 1 ? 0x3f800000u : 0x40000000u;
+  return __fadd_rn(__uint_as_float(one | (r >> 9)), -SCALE * (1.0f - 5.9604644775390625e-8f));
 }
 
 // Square root by the approximate instruction (relative error about one ulp).
@@ -343,13 +349,12 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // within a few ulp.
 __device__ __forceinline__ float2 nln_draw(uint4 r, float L00, float L10, float L11,
                                            float ln_mu, float ln_sigma) {
-  float u0 = unit_open(r.x), u1 = unit_open(r.y), u2 = unit_open(r.z), u3 = unit_open(r.w);
-  float ra = sqrt_approx(-2.0f * logf(u0));
+  float ra = sqrt_approx(-2.0f * logf(unit_open<1>(r.x)));
   float sa, ca;
-  sincospif(2.0f * u1, &sa, &ca);
-  float rb = sqrt_approx(-2.0f * logf(u2));
+  sincospif(unit_open<2>(r.y), &sa, &ca);
+  float rb = sqrt_approx(-2.0f * logf(unit_open<1>(r.z)));
   float sb, cb;
-  sincospif(2.0f * u3, &sb, &cb);
+  sincospif(unit_open<2>(r.w), &sb, &cb);
   float zn0 = ra * ca, zn1 = ra * sa;
   float g0 = __expf(ln_mu + ln_sigma * (rb * cb));
   float g1 = __expf(ln_mu + ln_sigma * (rb * sb));
@@ -1004,6 +1009,35 @@ __device__ __forceinline__ FF warp_sum_ff(FF a) {
     a = ff_sum(a, b);
   }
   return a;
+}
+
+// Sums of four float pairs over the 32 lanes at once: the first two rounds of
+// the butterfly each hand half of the pairs to the partner, so six pair sums
+// take the place of twenty.  Lane 8 q returns the sum of v[sum4_of_lane(8 q)],
+// formed in the order in which warp_sum_ff forms lane 0's (the lower lane's low
+// part first): the same bits.
+__device__ __forceinline__ FF ff_exchange_sum(FF a, FF b, int o, int lane) {
+  const bool up = lane & o;
+  const FF keep = up ? b : a, send = up ? a : b;
+  FF got;
+  got.hi = __shfl_xor_sync(0xffffffffu, send.hi, o);
+  got.lo = __shfl_xor_sync(0xffffffffu, send.lo, o);
+  return up ? ff_sum(got, keep) : ff_sum(keep, got);
+}
+__device__ __forceinline__ FF warp_sum_ff4(const FF (&v)[4], int lane) {
+  FF a = ff_exchange_sum(ff_exchange_sum(v[0], v[1], 16, lane),
+                         ff_exchange_sum(v[2], v[3], 16, lane), 8, lane);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    FF b;
+    b.hi = __shfl_xor_sync(0xffffffffu, a.hi, o);
+    b.lo = __shfl_xor_sync(0xffffffffu, a.lo, o);
+    a = ff_sum(a, b);
+  }
+  return a;
+}
+__device__ __forceinline__ int sum4_of_lane(int lane) {
+  return ((lane >> 4) & 1) | ((lane >> 2) & 2);
 }
 
 // Minimum of floats by an integer atomic: key(f) = ~u(f), u the

@@ -151,13 +151,12 @@ template <int MODEL, bool COST>
 __device__ void scan_trajectory(const CtrlDesc& D, int T, const float2* V, int vs,
                                 const float* __restrict__ x_init, float4* pose, int ps,
                                 const float2* __restrict__ Uf, const float2* __restrict__ Af,
-                                const float* __restrict__ xrf, FF& cost, int lane,
-                                float* x1 = nullptr) {
+                                const float* __restrict__ xrf, float sin0, float cos0, FF& cost,
+                                int lane, float* x1 = nullptr) {
   const float dt = D.dt;
   if constexpr (MODEL == 0) {
     float cth = x_init[2], cx = x_init[0], cy = x_init[1];
-    float cs_, cc_;
-    sincosf(cth, &cs_, &cc_);
+    float cs_ = sin0, cc_ = cos0;
     float lc = 0.0f;  // this lane's few stage terms, in FP32
     for (int t0 = 0; t0 < T; t0 += 32) {
       const int t = t0 + lane;
@@ -201,8 +200,7 @@ __device__ void scan_trajectory(const CtrlDesc& D, int T, const float2* V, int v
     // Ackermann (Eq. 14): speed -> heading (rate v tan(steer) / L) ->
     // (cos, sin) -> position, each a prefix sum over the segment's steps
     float cx = x_init[0], cy = x_init[1], cth = x_init[2], cv = x_init[3];
-    float cs_, cc_;
-    sincosf(cth, &cs_, &cc_);
+    float cs_ = sin0, cc_ = cos0;
     const float kth = D.k_turn * dt;  // 1 / L
     float lc = 0.0f;
     for (int t0 = 0; t0 < T; t0 += 32) {
@@ -262,8 +260,7 @@ __device__ void scan_trajectory(const CtrlDesc& D, int T, const float2* V, int v
     // sin) -> velocities (thrust m g + u_t) -> position
     float cx = x_init[0], cz = x_init[1], cth = x_init[2];
     float cvx = x_init[3], cvz = x_init[4];
-    float cs_, cc_;
-    sincosf(cth, &cs_, &cc_);
+    float cs_ = sin0, cc_ = cos0;
     float lc = 0.0f;
     for (int t0 = 0; t0 < T; t0 += 32) {
       const int t = t0 + lane;
@@ -323,8 +320,7 @@ __device__ void scan_trajectory(const CtrlDesc& D, int T, const float2* V, int v
   } else {
     float cy = x_init[0], cz = x_init[1], cph = x_init[2];
     float cvy = x_init[3], cvz = x_init[4], cw = x_init[5];
-    float cs_, cc_;
-    sincosf(cph, &cs_, &cc_);
+    float cs_ = sin0, cc_ = cos0;
     const float kw = D.k_turn * dt;  // arm / I
     float lc = 0.0f;
     for (int t0 = 0; t0 < T; t0 += 32) {
@@ -533,8 +529,10 @@ __device__ __forceinline__ void final_stage(const CtrlDesc& D, char* smem, const
   float* x1 = reinterpret_cast<float*>(smem + L.scH);  // per-sample sums are consumed
   if (tid < 32) {
     FF none = {0.0f, 0.0f};
-    scan_trajectory<MODEL, false>(D, T, Usf, 1, xi, pose_nom, 1, nullptr, nullptr, nullptr, none,
-                                  lane, x1);
+    float s0, c0_;
+    sincosf(xi[2], &s0, &c0_);
+    scan_trajectory<MODEL, false>(D, T, Usf, 1, xi, pose_nom, 1, nullptr, nullptr, nullptr, s0, c0_,
+                                  none, lane, x1);
   }
   __syncthreads();
   barrier_flat<GRID>(T * P, P, D.J, pose_nom, shp, obs4, D.h_eps, b_nom, tid, nthreads, gv);
@@ -705,11 +703,15 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
                          fminf(fmaxf(u.y + du.y, D.umin[1]), D.umax[1]));
     }
     __syncthreads();
+    const float* xi = reinterpret_cast<const float*>(smem + L.xi);
+    float sin0, cos0;
+    sincosf(xi[2], &sin0, &cos0);
     for (int s = warp; s < Sc; s += nwarps) {
       FF c = {0.0f, 0.0f};
-      scan_trajectory<MODEL, true>(D, T, V + s, Sc, reinterpret_cast<const float*>(smem + L.xi),
+      scan_trajectory<MODEL, true>(D, T, V + s, Sc, xi,
                                    pose + s, Sc, Uf, reinterpret_cast<const float2*>(smem + L.Af),
-                                   reinterpret_cast<const float*>(smem + L.xrf), c, lane);
+                                   reinterpret_cast<const float*>(smem + L.xrf), sin0, cos0, c,
+                                   lane);
       c = warp_sum_ff(c);
       if (lane == 0) {
         scH[s] = c.hi;
@@ -970,13 +972,48 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   }
 
   // ---- dynamics and stage/control costs: one warp per sample
-  for (int s = warp; s < S; s += nwarps) {
-    FF c = {0.0f, 0.0f};
-    scan_trajectory<MODEL, true>(D, T, V + s, SP, xi, pose + s, SP, Uf, Af, xrf, c, lane);
-    c = warp_sum_ff(c);
-    if (lane == 0) {
-      scH[s] = c.hi;
-      scL[s] = c.lo;
+  // (the persistent kernels add four samples' sums across the lanes together:
+  // six pair sums for twenty, 13.3 -> 13.0 ms for 512 controllers, 7.63 ->
+  // 7.24 ms for 96 served robots; the one-controller kernels, where a warp has
+  // one or two samples or the launch is one wave, lose 1 to 4 % to it)
+  {
+    if constexpr (BATCHED) {
+      float sin0, cos0;  // of the initial heading, the same for every sample
+      sincosf(xi[2], &sin0, &cos0);
+      for (int s0 = warp; s0 < S; s0 += 4 * nwarps) {
+        FF c4[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+          const int s = s0 + i * nwarps;
+          if (s >= S) break;
+          FF c = {0.0f, 0.0f};
+          scan_trajectory<MODEL, true>(D, T, V + s, SP, xi, pose + s, SP, Uf, Af, xrf, sin0, cos0,
+                                       c, lane);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (i == k) c4[k] = c;
+        }
+        __syncwarp();
+        const FF c = warp_sum_ff4(c4, lane);
+        const int s = s0 + sum4_of_lane(lane) * nwarps;
+        if ((lane & 7) == 0 && s < S) {
+          scH[s] = c.hi;
+          scL[s] = c.lo;
+        }
+      }
+    } else {
+      for (int s = warp; s < S; s += nwarps) {
+        float sin0, cos0;
+        sincosf(xi[2], &sin0, &cos0);
+        FF c = {0.0f, 0.0f};
+        scan_trajectory<MODEL, true>(D, T, V + s, SP, xi, pose + s, SP, Uf, Af, xrf, sin0, cos0, c,
+                                     lane);
+        c = warp_sum_ff(c);
+        if (lane == 0) {
+          scH[s] = c.hi;
+          scL[s] = c.lo;
+        }
+      }
     }
   }
   __syncthreads();
@@ -1013,24 +1050,55 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   // controller, so it cancels in the weights)
   float* relH = reinterpret_cast<float*>(smem + L.scH);
   float* relL = reinterpret_cast<float*>(smem + L.scL);
-  for (int s = warp; s < S; s += nwarps) {
-    FF b = {0.0f, 0.0f};
-    bool coll = false;
-    for (int t = lane; t < T; t += 32) {
-      const float2 v = uB[2 * (t * SP + s)];
-      const bool cl = __float_as_int(v.x) < 0;
-      ff_add_prod(b, cw[t], fabsf(v.x), v.y);
-      if (cl) ff_add(b, D.C_coll);
-      coll |= cl;
+  if constexpr (BATCHED) {
+    for (int s0 = warp; s0 < S; s0 += 4 * nwarps) {
+      FF b4[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+      unsigned hit = 0u;  // bit k: sample s0 + k nwarps collided
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int s = s0 + k * nwarps;
+        if (s >= S) break;
+        bool coll = false;
+        for (int t = lane; t < T; t += 32) {
+          const float2 v = uB[2 * (t * SP + s)];
+          const bool cl = __float_as_int(v.x) < 0;
+          ff_add_prod(b4[k], cw[t], fabsf(v.x), v.y);
+          if (cl) ff_add(b4[k], D.C_coll);
+          coll |= cl;
+        }
+        __syncwarp();
+        if (__any_sync(0xffffffffu, coll)) hit |= 1u << k;
+      }
+      const FF b = warp_sum_ff4(b4, lane);
+      const int k = sum4_of_lane(lane), s = s0 + k * nwarps;
+      if ((lane & 7) == 0 && s < S) {
+        FF c = {scH[s], scL[s]};
+        c = ff_norm(ff_sum(c, b));
+        relH[s] = c.hi;
+        relL[s] = c.lo;
+        collf[s] = (hit >> k) & 1u;
+      }
     }
-    b = warp_sum_ff(b);
-    coll = __any_sync(0xffffffffu, coll);
-    if (lane == 0) {
-      FF c = {scH[s], scL[s]};
-      c = ff_norm(ff_sum(c, b));
-      relH[s] = c.hi;
-      relL[s] = c.lo;
-      collf[s] = coll ? 1 : 0;
+  } else {
+    for (int s = warp; s < S; s += nwarps) {
+      FF b = {0.0f, 0.0f};
+      bool coll = false;
+      for (int t = lane; t < T; t += 32) {
+        const float2 v = uB[2 * (t * SP + s)];
+        const bool cl = __float_as_int(v.x) < 0;
+        ff_add_prod(b, cw[t], fabsf(v.x), v.y);
+        if (cl) ff_add(b, D.C_coll);
+        coll |= cl;
+      }
+      b = warp_sum_ff(b);
+      coll = __any_sync(0xffffffffu, coll);
+      if (lane == 0) {
+        FF c = {scH[s], scL[s]};
+        c = ff_norm(ff_sum(c, b));
+        relH[s] = c.hi;
+        relL[s] = c.lo;
+        collf[s] = coll ? 1 : 0;
+      }
     }
   }
   __syncthreads();
