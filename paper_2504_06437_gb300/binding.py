@@ -20,7 +20,8 @@ _SOURCES = ["csrc/dbasmppi.cu", "csrc/k_step_u.cu", "csrc/k_step_q.cu", "csrc/k_
             "csrc/k_step_a_r80.cu", "csrc/k_step_p_r80.cu", "csrc/k_step_u_sgf.cu",
             "csrc/k_step_q_sgf.cu", "csrc/k_step_a_sgf.cu", "csrc/k_step_p_sgf.cu",
             "csrc/k_step_u_grid.cu", "csrc/k_step_q_grid.cu", "csrc/k_step_a_grid.cu",
-            "csrc/k_step_p_grid.cu", "csrc/k_batch.cu", "csrc/k_batch_all.cu"]
+            "csrc/k_step_p_grid.cu", "csrc/k_step_u_far.cu", "csrc/k_step_q_far.cu",
+            "csrc/k_step_a_far.cu", "csrc/k_step_p_far.cu", "csrc/k_batch.cu", "csrc/k_batch_all.cu"]
 _DEPS = _SOURCES + ["csrc/mppi_device.cuh", "csrc/mppi_tile.cuh", "csrc/kernels.cuh"]
 HEADER = os.path.join(_ROOT, "include", "dbasmppi.h")
 

@@ -78,14 +78,14 @@ __global__ void draws_kernel(int K, int T, uint32_t k0, uint32_t k1, uint32_t it
 
 using StepFn = void (*)(CtrlDesc, const double*, const double*);
 
-StepFn pick_kernel(int model, int npos, bool r80) {
-  // [model][points 8 / 14][register form 96 / 80]
-  static const StepFn table[MPPI_NUM_MODELS][2][2] = {
-      {{step_u8, step_u8_r80}, {step_u14, step_u14_r80}},
-      {{step_q8, step_q8_r80}, {step_q14, step_q14_r80}},
-      {{step_a8, step_a8_r80}, {step_a14, step_a14_r80}},
-      {{step_p8, step_p8_r80}, {step_p14, step_p14_r80}}};
-  return table[model][npos == 14 ? 1 : 0][r80 ? 1 : 0];
+StepFn pick_kernel(int model, int npos, bool r80, bool far) {
+  // [model][points 8 / 14][96 registers, 96 with far-field cells, 80 (with them)]
+  static const StepFn table[MPPI_NUM_MODELS][2][3] = {
+      {{step_u8, step_u8_far, step_u8_r80}, {step_u14, step_u14_far, step_u14_r80}},
+      {{step_q8, step_q8_far, step_q8_r80}, {step_q14, step_q14_far, step_q14_r80}},
+      {{step_a8, step_a8_far, step_a8_r80}, {step_a14, step_a14_far, step_a14_r80}},
+      {{step_p8, step_p8_far, step_p8_r80}, {step_p14, step_p14_far, step_p14_r80}}};
+  return table[model][npos == 14 ? 1 : 0][r80 ? 2 : far ? 1 : 0];
 }
 
 // Forms of the step kernels beyond the plain one (96-register form, separate
@@ -93,13 +93,17 @@ StepFn pick_kernel(int model, int npos, bool r80) {
 // smooths the update (Savitzky-Golay), kFormGrid adds the grid map's barrier
 // terms and smooths when asked.
 constexpr int kFormPlain = 0, kFormSgf = 1, kFormGrid = 2;
-StepFn pick_form_kernel(int form, int model, int npos) {
-  static const StepFn table[2][MPPI_NUM_MODELS][2] = {
-      {{step_u8_sgf, step_u14_sgf}, {step_q8_sgf, step_q14_sgf},
-       {step_a8_sgf, step_a14_sgf}, {step_p8_sgf, step_p14_sgf}},
-      {{step_u8_grid, step_u14_grid}, {step_q8_grid, step_q14_grid},
-       {step_a8_grid, step_a14_grid}, {step_p8_grid, step_p14_grid}}};
-  return table[form == kFormGrid ? 1 : 0][model][npos == 14 ? 1 : 0];
+StepFn pick_form_kernel(int form, int model, int npos, bool far) {
+  static const StepFn table[2][MPPI_NUM_MODELS][2][2] = {
+      {{{step_u8_sgf, step_u8_sgf_far}, {step_u14_sgf, step_u14_sgf_far}},
+       {{step_q8_sgf, step_q8_sgf_far}, {step_q14_sgf, step_q14_sgf_far}},
+       {{step_a8_sgf, step_a8_sgf_far}, {step_a14_sgf, step_a14_sgf_far}},
+       {{step_p8_sgf, step_p8_sgf_far}, {step_p14_sgf, step_p14_sgf_far}}},
+      {{{step_u8_grid, step_u8_grid_far}, {step_u14_grid, step_u14_grid_far}},
+       {{step_q8_grid, step_q8_grid_far}, {step_q14_grid, step_q14_grid_far}},
+       {{step_a8_grid, step_a8_grid_far}, {step_a14_grid, step_a14_grid_far}},
+       {{step_p8_grid, step_p8_grid_far}, {step_p14_grid, step_p14_grid_far}}}};
+  return table[form == kFormGrid ? 1 : 0][model][npos == 14 ? 1 : 0][far ? 1 : 0];
 }
 
 // World points a barrier thread holds: whole units of P points each; the
@@ -267,29 +271,30 @@ int max_smem_optin() {
 // (the allocation-free entry point calls this every step).
 struct PickMemo {
   int model, npos, threads, smem, nTiles, chunk;
+  bool far;
   StepFn fn;
 };
 std::mutex g_pick_mu;
-bool g_step_attr[kMaxPickDevices][MPPI_NUM_MODELS] = {};
-bool g_form_attr[kMaxPickDevices][2][MPPI_NUM_MODELS] = {};
+bool g_step_attr[kMaxPickDevices][MPPI_NUM_MODELS][2] = {};
+bool g_form_attr[kMaxPickDevices][2][MPPI_NUM_MODELS][2] = {};
 PickMemo g_pick_memo[kMaxPickDevices] = {};
 
-int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, int form,
+int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, int form, bool far,
                        StepFn* out, int* chunk) {
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxPickDevices) return fail(MPPI_EINVAL, "device %d out of range", dev);
   std::lock_guard<std::mutex> lock(g_pick_mu);
   if (form != kFormPlain) {
-    bool& done = g_form_attr[dev][form == kFormGrid ? 1 : 0][model];
+    bool& done = g_form_attr[dev][form == kFormGrid ? 1 : 0][model][far ? 1 : 0];
     if (!done) {
       const int lim = max_smem_optin();
       for (int np : {8, 14})
-        CK(cudaFuncSetAttribute(pick_form_kernel(form, model, np),
+        CK(cudaFuncSetAttribute(pick_form_kernel(form, model, np, far),
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
       done = true;
     }
-    *out = pick_form_kernel(form, model, npos);
+    *out = pick_form_kernel(form, model, npos, far);
     int occ = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, *out, threads, smem));
     *chunk = chunk_of(nTiles, (long)std::max(occ, 1) * num_sms());
@@ -297,28 +302,28 @@ int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, i
   }
   // only this model's kernels: with lazy module loading, touching a kernel
   // loads its module, and the models a process never steps stay unloaded
-  if (!g_step_attr[dev][model]) {
+  if (!g_step_attr[dev][model][far ? 1 : 0]) {
     const int lim = max_smem_optin();
     for (int np : {8, 14})
       for (bool r80 : {false, true})
-        CK(cudaFuncSetAttribute(pick_kernel(model, np, r80),
+        CK(cudaFuncSetAttribute(pick_kernel(model, np, r80, far),
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    g_step_attr[dev][model] = true;
+    g_step_attr[dev][model][far ? 1 : 0] = true;
   }
   PickMemo& m = g_pick_memo[dev];
-  if (m.fn && m.model == model && m.npos == npos && m.threads == threads && m.smem == smem &&
+  if (m.fn && m.far == far && m.model == model && m.npos == npos && m.threads == threads && m.smem == smem &&
       m.nTiles == nTiles) {
     *out = m.fn;
     *chunk = m.chunk;
     return MPPI_OK;
   }
-  const StepFn hi = pick_kernel(model, npos, false), lo = pick_kernel(model, npos, true);
+  const StepFn hi = pick_kernel(model, npos, false, far), lo = pick_kernel(model, npos, true, far);
   int occ_hi = 0, occ_lo = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_hi, hi, threads, smem));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_lo, lo, threads, smem));
   const StepFn fn = (occ_lo > occ_hi && (long)nTiles > (long)occ_hi * num_sms()) ? lo : hi;
   *chunk = chunk_of(nTiles, (long)std::max(fn == lo ? occ_lo : occ_hi, 1) * num_sms());
-  m = PickMemo{model, npos, threads, smem, nTiles, *chunk, fn};
+  m = PickMemo{model, npos, threads, smem, nTiles, *chunk, far, fn};
   *out = fn;
   return MPPI_OK;
 }
@@ -687,7 +692,8 @@ int mppi_create_tiled(const mppi_params* p, const double* u_init, const mppi_til
   c->last = c->own;
   fill_desc(c);
   rc = choose_step_kernel(p->model, c->tl.positions_per_thread, c->tl.threads, c->smem, nTiles,
-                          p->sgf_window > 0 ? kFormSgf : kFormPlain, &c->fn, &c->D.chunk);
+                          p->sgf_window > 0 ? kFormSgf : kFormPlain, c->nc > 0, &c->fn,
+                          &c->D.chunk);
   if (rc) {
     free_ctx(c);
     return rc;
@@ -751,7 +757,7 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   StepFn fn = nullptr;
   int chunk = 1;
   rc = choose_step_kernel(c->p.model, t.positions_per_thread, t.threads, smem, c->D.nTiles,
-                          step_form(c), &fn, &chunk);
+                          step_form(c), nc > 0, &fn, &chunk);
   if (rc) return rc;
   c->tl = t;
   c->smem = smem;
@@ -790,8 +796,8 @@ int mppi_set_grid(mppi_ctx* c, const float* sdf, int32_t nx, int32_t ny, double 
   int chunk = 1;
   int rc = choose_step_kernel(c->p.model, c->tl.positions_per_thread, c->tl.threads, c->smem,
                               c->D.nTiles,
-                              off ? (c->p.sgf_window > 0 ? kFormSgf : kFormPlain) : kFormGrid, &fn,
-                              &chunk);
+                              off ? (c->p.sgf_window > 0 ? kFormSgf : kFormPlain) : kFormGrid,
+                              c->nc > 0, &fn, &chunk);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->last));  // no step in flight reads the old map
   float* nb = nullptr;
@@ -976,7 +982,7 @@ int mppi_get_tiling(mppi_ctx* c, mppi_tiling* t, int32_t* n_ctas) {
 int mppi_get_kernel_regs(mppi_ctx* c, int32_t* regs_cap) {
   if (!c) return fail(MPPI_ESTATE, "context is NULL");
   if (!regs_cap) return fail(MPPI_EINVAL, "regs_cap is NULL");
-  const bool r80 = c->fn == pick_kernel(c->p.model, c->tl.positions_per_thread, true);
+  const bool r80 = c->fn == pick_kernel(c->p.model, c->tl.positions_per_thread, true, c->nc > 0);
   *regs_cap = r80 ? DBM_STEP_MAXNREG_R80 : DBM_STEP_MAXNREG;
   return MPPI_OK;
 }
@@ -1183,7 +1189,7 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   StepFn fn = nullptr;  // picked before anything is launched
   int chunk = 1;
   rc = choose_step_kernel(p->model, c.tl.positions_per_thread, c.tl.threads, c.smem, nTiles,
-                          p->sgf_window > 0 ? kFormSgf : kFormPlain, &fn, &chunk);
+                          p->sgf_window > 0 ? kFormSgf : kFormPlain, c.nc > 0, &fn, &chunk);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   c.d_U = d_U;

@@ -5,6 +5,7 @@
 
 namespace dbm {
 
+// (two CTAs per SM: without the bound the allocation rises to 255 registers)
 __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const CtrlDesc* __restrict__ descs,
                                                               unsigned char* stage,
                                                               double* __restrict__ u0_out) {

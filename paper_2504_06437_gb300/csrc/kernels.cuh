@@ -100,6 +100,31 @@ __global__ void step_p8_grid(const __grid_constant__ CtrlDesc D, const double* _
 __global__ void step_p14_grid(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,
                               const double* __restrict__ xref);
 
+// The 96-register forms with the far-field cells compiled in (suffix _far),
+// launched only for problems that use them.
+#define DBM_STEP_FAR(m)                                                                          \
+  __global__ void step_##m##8_far(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,  \
+                                  const double* __restrict__ xref);                               \
+  __global__ void step_##m##14_far(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0, \
+                                   const double* __restrict__ xref);                              \
+  __global__ void step_##m##8_sgf_far(const __grid_constant__ CtrlDesc D,                         \
+                                      const double* __restrict__ x0,                              \
+                                      const double* __restrict__ xref);                           \
+  __global__ void step_##m##14_sgf_far(const __grid_constant__ CtrlDesc D,                        \
+                                       const double* __restrict__ x0,                             \
+                                       const double* __restrict__ xref);                          \
+  __global__ void step_##m##8_grid_far(const __grid_constant__ CtrlDesc D,                        \
+                                       const double* __restrict__ x0,                             \
+                                       const double* __restrict__ xref);                          \
+  __global__ void step_##m##14_grid_far(const __grid_constant__ CtrlDesc D,                       \
+                                        const double* __restrict__ x0,                            \
+                                        const double* __restrict__ xref);
+DBM_STEP_FAR(u)
+DBM_STEP_FAR(q)
+DBM_STEP_FAR(a)
+DBM_STEP_FAR(p)
+#undef DBM_STEP_FAR
+
 // Batched step: persistent CTAs pull (controller, first tile) work items.
 struct WorkItem {
   int ctrl;  // index into the step table
@@ -272,14 +297,14 @@ __device__ __forceinline__ void serve_body(const CtrlDesc* __restrict__ descs, c
 }
 
 // Body of the one-controller step kernels.
-template <int MODEL, int NPOS, bool SGF = false, bool GRID = false>
+template <int MODEL, int NPOS, bool SGF = false, bool GRID = false, bool FAR = false>
 __device__ __forceinline__ void step_body(const CtrlDesc& D, const double* __restrict__ x0,
                                           const double* __restrict__ xref) {
   TileScratch& ts = tile_scratch();
   if (threadIdx.x == 0) mbar_init(&ts.mbar);
   __syncthreads();
   uint32_t phase = 0u;
-  run_tile_inl<MODEL, NPOS, false, SGF, GRID>(D, blockIdx.x * D.chunk, D.chunk, x0, xref, phase);
+  run_tile_inl<MODEL, NPOS, false, SGF, GRID, FAR>(D, blockIdx.x * D.chunk, D.chunk, x0, xref, phase);
 }
 
 }  // namespace dbm

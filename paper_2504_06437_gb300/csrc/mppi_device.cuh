@@ -1,8 +1,8 @@
 // Device side of the DBaS-Log-MPPI step (arXiv 2504.06437), sm_103a.
 //
 // One controller's K samples are cut into tiles of S <= 32 samples; a CTA
-// processes one tile (plain step: one CTA per tile; batched step: persistent
-// CTAs pull (controller, tile) work items).  Per tile:
+// processes one tile or a few in a row (batched step: persistent CTAs pull
+// (controller, first tile) work items).  Per tile:
 //   noise      all threads draw the NLN perturbations of every (sample, step)
 //              (Eq. 11) from Philox4x32-10 with counter (k, t, iter) -- no
 //              noise crosses HBM -- and keep the clamped controls v = u + du;
@@ -18,14 +18,17 @@
 //              set from shared memory (broadcast reads), evaluates two points
 //              per packed two-lane FP32 instruction, adds two obstacles per
 //              approximate reciprocal, and sums each unit's points exactly
-//              into a float pair, written over the unit's pose;
+//              into a float pair, written over the unit's pose; in large
+//              problems only the obstacles near a cell of poses are streamed
+//              and the others enter through one polynomial per cell (FarCell);
 //   costs      one warp per sample adds the barrier-state and collision costs;
 //   partials   the tile's minimum cost, its exponentiated weights, their sum Z
 //              and the 2T weighted column sums of the perturbations (Eq. 4);
 //   merge      the last tile to finish (a ticket per group of tiles) merges
 //              the partials log-sum-exp style against the exact minimum over
-//              the tiles, then runs the final stage (U*, nominal rollout, S_e,
-//              shift).
+//              the tiles, sums the barriers of the samples that carry the
+//              weights directly once more if cells were used, then runs the
+//              final stage (U*, nominal rollout, S_e, shift).
 // The one-controller kernels exist in a 96- and an 80-register form (the
 // host picks per launch); the batch kernel's tiles take a padded row stride
 // and the one-batch merge (BATCHED in run_tile).  All forms give the same
@@ -187,10 +190,10 @@ __host__ __device__ inline int merge_buf_bytes(int ncol, int nthreads) {
 // the limit, and 2^-9 of that half way in.  A trajectory tile is small beside
 // the world: of 200 obstacles about 10 are near a cell of the 65536-sample
 // unicycle, of 500 about 40 near one of the crowded quadrotor.  Without and
-// with cells, a whole call: unicycle K 65536, T 100, J 200 608 and 365 us;
-// quadrotor K 32768, T 100, J 500, P 7 3090 and 830 us; vehicle K 9973, T 73,
-// J 117, P 8 305 and 162 us; 512 mixed controllers in one launch 29.2 and
-// 13.8 ms.  Degree 8 against 6 and 10, and cells of 1024 points against one or
+// with cells, a whole call, all else as it was then: unicycle K 65536, T 100, J 200
+// 608 and 365 us; quadrotor K 32768, T 100, J 500, P 7 3090 and 830 us; vehicle
+// K 9973, T 73, J 117, P 8 305 and 162 us; 512 mixed controllers in one launch
+// 29.2 and 13.8 ms.  Degree 8 against 6 and 10, and cells of 1024 points against one or
 // sixteen per tile, come from counting the operations over the presets'
 // rollouts (least at 8 and 800 to 2800 points).
 constexpr int kFarN = 8;
@@ -216,7 +219,7 @@ __host__ __device__ inline int far_list_cap(int J) {
 // presets' densities give) and its share of the set-up.  The line of 4e7 over
 // the whole step is about 8 us of the GPU, what the last CTA's second look
 // (refine_samples) takes when it is needed: the quadrotor at K 4096, T 50,
-// J 40 (2e7) takes 71.5 us a call without cells, 72 to 80 us with them; at
+// J 40 (2e7) took 71.5 us a call without cells, 72 to 80 us with them; at
 // K 8192, T 40, J 60 (7e7) 104 us without, 86 to 92 us with them.
 constexpr int kFarCellPoints = 1024;
 constexpr float kFarMinSaved = 4.0e7f;
@@ -776,7 +779,7 @@ struct BoolC {
 // has h >= h_eps all over its cell).  A lane reads the poses of its units
 // before it writes their sums, so uB may overlay pose.  GRID: each point also
 // adds the grid map's term (grid_h) and counts its h in the collision test.
-template <int NPOS, bool BATCHED, bool GRID = false>
+template <int NPOS, bool BATCHED, bool FAR, bool GRID = false>
 __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, const float4* pose,
                                               const float2* __restrict__ shp,
                                               const float4* __restrict__ obs4, float h_eps,
@@ -833,8 +836,11 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
       }
     };
     // obstacles in pairs: 1/h1 + 1/h2 = (h1 + h2) / (h1 h2), one reciprocal
-    // for two terms (h1 h2 stays finite for |p - c| < 4e9 m and h_eps >= 1e-18);
-    // with more points per thread the pair's temporaries would not fit
+    // for two terms (h1 h2 stays finite for |p - c| < 4e9 m and h_eps >= 1e-18).
+    // At 14 points per lane only the lists of near obstacles do so (a call at
+    // K 32768, J 500 829 -> 786 us: one reciprocal per pair of point and obstacle
+    // binds the special-function pipe); the loop over all obstacles keeps one
+    // each, whose sums barrier_refine forms bit for bit.
     auto two = [&](const float4 o, const float4 q, auto paired) {
       if constexpr (decltype(paired)::value) {
         const float2 nox = make_float2(-o.x, -o.x), noy = make_float2(-o.y, -o.y);
@@ -860,18 +866,23 @@ __device__ __forceinline__ void barrier_units(int nunits, int S, int P, int J, c
         one(q);
       }
     };
-    const int c = nc > 0 ? g * nc / NG : 0;
-    int nn = nc > 0 ? cells[c].n_near : -1;
-    if (nn >= 0) {
-      far_eval<NP2>(cells + c, X2, Y2, acc2);
-      const unsigned short* l = lists + c * far_list_cap(J);
-      int j = 0;
-      for (; j + 1 < nn; j += 2) {
-        const unsigned jj = *reinterpret_cast<const unsigned*>(l + j);
-        two(obs4[jj & 0xffffu], obs4[jj >> 16], BoolC<true>());
+    bool direct = true;
+    if constexpr (FAR) {
+      const int c = nc > 0 ? g * nc / NG : 0;
+      const int nn = nc > 0 ? cells[c].n_near : -1;
+      if (nn >= 0) {
+        direct = false;
+        far_eval<NP2>(cells + c, X2, Y2, acc2);
+        const unsigned short* l = lists + c * far_list_cap(J);
+        int j = 0;
+        for (; j + 1 < nn; j += 2) {
+          const unsigned jj = *reinterpret_cast<const unsigned*>(l + j);
+          two(obs4[jj & 0xffffu], obs4[jj >> 16], BoolC<true>());
+        }
+        if (j < nn) one(obs4[l[j]]);
       }
-      if (j < nn) one(obs4[l[j]]);
-    } else {
+    }
+    if (direct) {
       int j = 0;
       for (; j + 1 < J; j += 2) two(obs4[j], obs4[j + 1], BoolC<(NPOS <= 8)>());
       if (j < J) one(obs4[j]);

@@ -665,8 +665,10 @@ __device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, 
 // is summed.  Taking those few again leaves the polynomial no say in it: they
 // end with the bits of the direct evaluation.  They are drawn and rolled out
 // anew (the generator is counter based).  The last CTA runs this alone, a
-// chain of latencies (about 8 us); out of line, so that its registers leave
-// the tile's code as it is.
+// chain of latencies (list 2.5, draws 1, rollout 2, barrier 2 to 20, costs 1,
+// columns 1 us); out of line, so that its registers leave the tile's code as
+// it is: as a second round of the tile's own code it took the batch kernel
+// from 13.4 to 14.4 ms.
 template <int MODEL, int NPOS, bool BATCHED, bool GRID>
 __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const CtrlDesc& D = BATCHED ? tile_desc() : D_;
@@ -775,12 +777,16 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
 // The batch kernels carry it, and the one-controller kernels have a form
 // with it and one without, so that controllers that do not smooth run code
 // with no trace of it.
+// FAR: far-field cells are compiled in (taken when D.nc is set).  The
+// 96-register one-controller kernels have a form with them and one without:
+// a small step after an L2 flush fetches its code from memory, and with the
+// cells' code in the kernel, though not taken, it was 3 to 7 us longer.
 // The one-controller kernels inline the body (run_tile_inl), so the
 // descriptor stays the kernel's own parameter: its fields are read from the
 // parameter bank, and no store in the body can alias them.  The batch
 // kernels call it out of line (run_tile), which keeps their four-model
 // switch small.
-template <int MODEL, int NPOS, bool BATCHED, bool SGF = BATCHED, bool GRID = false>
+template <int MODEL, int NPOS, bool BATCHED, bool SGF = BATCHED, bool GRID = false, bool FAR = true>
 __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int count,
                                              const double* __restrict__ x0g,
                                              const double* __restrict__ xrefg, uint32_t& mbar_phase,
@@ -1021,26 +1027,28 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   // ---- far-field cells: one warp sets up one cell of the tile's units
   FarCell* cells = reinterpret_cast<FarCell*>(smem + L.cell);
   unsigned short* lists = reinterpret_cast<unsigned short*>(smem + L.list);
-  const int nc = D.nc;
-  if (nc > 0) {
-    if (warp < nc) {
-      const int gsz = 32 * (NPOS / P), NG = (T * S + gsz - 1) / gsz;
-      // the groups g of cell c are those with g nc / NG = c
-      const int g0 = (warp * NG + nc - 1) / nc, g1 = ((warp + 1) * NG + nc - 1) / nc;
-      far_setup<BATCHED>(L.cell + warp * (int)sizeof(FarCell), L.list + 2 * warp * far_list_cap(J),
-                         L.pose, L.obs4, g0 * gsz, min(g1 * gsz, T * S), S, J, D.r_body, D.h_eps,
-                         lane);
+  const int nc = FAR ? D.nc : 0;
+  if constexpr (FAR) {
+    if (nc > 0) {
+      if (warp < nc) {
+        const int gsz = 32 * (NPOS / P), NG = (T * S + gsz - 1) / gsz;
+        // the groups g of cell c are those with g nc / NG = c
+        const int g0 = (warp * NG + nc - 1) / nc, g1 = ((warp + 1) * NG + nc - 1) / nc;
+        far_setup<BATCHED>(L.cell + warp * (int)sizeof(FarCell), L.list + 2 * warp * far_list_cap(J),
+                           L.pose, L.obs4, g0 * gsz, min(g1 * gsz, T * S), S, J, D.r_body, D.h_eps,
+                           lane);
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
 
   // ---- fused barrier over all (step, sample) units, sums over the poses
   if constexpr (GRID) {
     const GridView gv = grid_shared();
-    barrier_units<NPOS, BATCHED, true>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid,
+    barrier_units<NPOS, BATCHED, FAR, true>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid,
                                        nthreads, nc, cells, lists, &gv);
   } else {
-    barrier_units<NPOS, BATCHED>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid, nthreads,
+    barrier_units<NPOS, BATCHED, FAR>(T * S, S, P, J, pose, shp, obs4, D.h_eps, uB, 2, tid, nthreads,
                                  nc, cells, lists);
   }
   __syncthreads();
@@ -1192,8 +1200,10 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
                              nthreads);
   }
   // (one sample with all but 1 / kRefShare of the weight needs no second look)
-  if (D.nc > 0 && ts.Z.hi > 1.0f + 1.0f / kRefShare)
-    refine_samples<MODEL, NPOS, BATCHED, GRID>(D);
+  if constexpr (FAR) {
+    if (D.nc > 0 && ts.Z.hi > 1.0f + 1.0f / kRefShare)
+      refine_samples<MODEL, NPOS, BATCHED, GRID>(D);
+  }
   if constexpr (SGF) {
     if (D.sgf_wp)
       sgf_columns(D.cw + sgf_table_offset(T), D.sgf_wp & 0xff, T, col_hi, col_lo,
