@@ -442,6 +442,7 @@ void free_ctx(mppi_ctx* c) {
 // From 12 on, S avoids multiples of 4: the scans read a sample's steps S
 // words of 8 or 16 bytes apart, and those strides fold the lanes onto a few
 // shared-memory banks (S 32 against 31 is the unicycle's 335 against 286).
+constexpr int kServeStatic = 16 << 10;  // bytes the serving kernel holds beyond its tile, at most
 constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31;
 void default_shape(int K, int sms, int* S, int* threads) {
   if (K <= 32 * sms) {
@@ -491,15 +492,16 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
     const int GT = group_size(nTiles);
     const int nGroups = (nTiles + GT - 1) / GT;
     const int nscl = GT > nGroups ? GT : nGroups;
-    // with far-field cells where they fit, else without them
-    const int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads);
-    SmemLayout L = smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, nc,
-                               batched);
+    // with far-field cells where they fit the persistent kernels' tile too,
+    // whose rows are wider and whose serving form has 13 KB of its own: a
+    // controller takes them alone, batched and served or not at all
+    int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads);
+    if (nc > 0 && smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, nc,
+                              true).total > limit - kServeStatic)
+      nc = 0;
     *nc_out = nc;
-    if (L.total > limit && nc > 0) {
-      L = smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, 0, batched);
-      *nc_out = 0;
-    }
+    const SmemLayout L = smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl,
+                                     t.threads / 32, nc, batched);
     if (L.total <= limit) {
       *smem_out = L.total;
       break;

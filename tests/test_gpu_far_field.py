@@ -103,3 +103,28 @@ def test_far_field_costs_match_the_oracle(case, orc):
     assert np.abs(dbg["Ustar"] - ro["Ustar"]).max() <= bound
     for k in ("costs", "coll", "Ustar"):               # the same bits again
         assert np.array_equal(dbg[k], again[k])
+
+
+@pytest.mark.parametrize("T", [200, 240])
+def test_served_tiles_near_the_shared_memory_limit(T, orc):
+    """Tiles of 32 samples of a long horizon fill the serving kernel's shared
+    memory; with no room for cells beside them the request still runs, and
+    gives the bits of the same shape alone."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2504_06437_gb300 import binding
+    w = _uni(2048, T, 400, 63.0, seed=8)
+    x, xref = w.x_start, w.reference(w.x_start)
+    with binding.Server(1, 256 << 20) as s:
+        s.set_policy(small_ops_max=0.0, device_queue=True)
+        r = s.join(w.params, w.obstacles)
+        s.submit(r, x, xref)
+        done = []
+        while not done:
+            done = s.poll()
+    assert done[0][4] == 0
+    with binding.Controller(w.params, tiling=dict(samples_per_cta=32, threads=256, positions_per_thread=0)) as g:
+        g.set_obstacles(w.obstacles)
+        g.step(x, xref)
+        assert np.array_equal(done[0][1], g.get_control())
