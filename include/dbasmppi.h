@@ -19,7 +19,10 @@
  *   - A context is used from one host thread at a time.
  *   - "stream" is a cudaStream_t passed as void*; NULL selects the
  *     context's own stream.  mppi_step*() only enqueue work; the mppi_get_*()
- *     calls synchronise with the stream of the last step.
+ *     calls wait for the last step's results, and all but mppi_get_control()
+ *     synchronise with its stream.  A step on another stream than the step
+ *     before it runs after it once mppi_get_control() has returned that
+ *     step's results.
  *   - Device work that times out on a bounded wait reports MPPI_ETIMEOUT at
  *     the next mppi_get_*() call.
  */

@@ -368,6 +368,7 @@ struct mppi_ctx {
   cudaEvent_t in_ev[2] = {nullptr, nullptr};
   bool in_ev_pending[2] = {false, false};
   int in_next = 0;
+  cudaEvent_t order = nullptr;  // in_ev of the last step, when it came from mppi_step
   DevState* h_st = nullptr; // pinned readback
   double* h_U = nullptr;    // pinned readback
   HostOut* h_out = nullptr;      // mapped mirror of u0, status and the sequence, written by the step
@@ -843,8 +844,38 @@ namespace {
 // reads the control on the host); the device-input entry point leaves it
 // out, since the system-scope fence adds the host link's round trip to the
 // kernel's retirement.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+// mppi_get_control can return while the final stage of the step it reports
+// still writes the state that the next step reads.  The stream of that step
+// orders the two; a step on another stream waits for its event.  A stream
+// that is being captured cannot wait for an event from outside the capture,
+// and the graph may be launched on any stream: there the host waits.
+// (cudaStreamPerThread is one handle for the streams of several threads.)
+int order_step(mppi_ctx* c, cudaStream_t s) {
+  if (!c->order) return MPPI_OK;
+  if (capturing(s)) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaEventSynchronize(c->order);
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    CK(e);
+  } else if (s != c->last || s == cudaStreamPerThread) {
+    CK(cudaStreamWaitEvent(s, c->order, 0));
+  }
+  return MPPI_OK;
+}
+
 int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream, bool mirror) {
   cudaStream_t s = stream ? (cudaStream_t)stream : c->own;
+  if (const int rc = order_step(c, s)) return rc;
   if (mirror) {
     c->fn<<<(c->D.nTiles + c->D.chunk - 1) / c->D.chunk, c->tl.threads, c->smem, s>>>(c->D, x0, xref);
   } else {
@@ -854,6 +885,7 @@ int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream,
   }
   CK(cudaGetLastError());
   c->last = s;
+  c->order = nullptr;
   c->stepped = true;
   c->mirrored = c->mirror_U = mirror;
   ++c->iter;
@@ -886,6 +918,7 @@ int mppi_step(mppi_ctx* c, const double* x0, const double* xref, void* stream) {
   const int rc = launch_step(c, c->h_in_dev[b], c->h_in_dev[b] + n, s, true);
   if (rc) return rc;
   CK(cudaEventRecord(c->in_ev[b], s));
+  if (!capturing(s)) c->order = c->in_ev[b];
   c->in_ev_pending[b] = true;
   c->in_next = b ^ 1;
   return MPPI_OK;
