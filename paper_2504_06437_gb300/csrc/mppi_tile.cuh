@@ -886,10 +886,11 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
 #else
     const double* raw = D.obst;
 #endif
-    // the raw (region) and converted (obs4) areas are distinct
+    // the raw (region) and converted (obs4) areas are distinct; only r^2
+    // enters h, so a radius from device memory may carry either sign
     for (int j = tid; j < J; j += nthreads) {
       double cx = raw[3 * j], cy = raw[3 * j + 1], r = raw[3 * j + 2];
-      obs4[j] = make_float4((float)(cx - ox), (float)(cy - oy), -(float)(r * r), (float)r);
+      obs4[j] = make_float4((float)(cx - ox), (float)(cy - oy), -(float)(r * r), fabsf((float)r));
     }
   }
   __syncthreads();
