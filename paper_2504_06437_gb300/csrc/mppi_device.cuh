@@ -674,7 +674,9 @@ __device__ __noinline__ void far_setup(int cell_off, int list_off, int pose_off,
   for (int i = 0; i < 48; ++i) acc[i] = 0.0f;
   for (int j = lane; j < J; j += 32) {
     float dx, dy, H;
-    if (!far(j, dx, dy, H)) continue;
+    // (an obstacle so far away that H overflows, as pads a set of fixed size,
+    // adds nothing; its offset times 1 / H = 0 would be no number)
+    if (!far(j, dx, dy, H) || H > 3.0e38f) continue;
     const float q = 1.0f / H, g = -2.0f * R * q;
     const float ax = g * dx, ay = g * dy, b = -R * R * q;
     float r0[kFarN + 1], r1[kFarN + 1];  // rows n - 1 and n

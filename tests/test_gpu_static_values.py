@@ -48,3 +48,17 @@ def test_a_radius_counts_by_its_square(model, J):
     minus = w.obstacles * np.array([1.0, 1.0, -1.0])
     for a, b in zip(_static(w, w.obstacles), _static(w, minus)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("where", [np.inf, -np.inf, 1e25, 1e300])
+def test_an_obstacle_out_of_sight_adds_nothing(where):
+    """A set padded to a fixed size with obstacles far beyond anything, at 14
+    points per lane (one reciprocal per obstacle, which any distance suits)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    w = _world("quad2d", 61)
+    pad = np.concatenate([w.obstacles, np.tile([[where, 0.0, 0.0]], (3, 1))])
+    a, b = _static(w, w.obstacles), _static(w, pad)
+    assert np.isfinite(b[0]).all()
+    assert (np.abs(a[0] - b[0]) <= 2e-5 * np.maximum(np.abs(a[0]), 1.0)).all()
