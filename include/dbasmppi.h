@@ -196,11 +196,12 @@ int mppi_step_device(mppi_ctx* c, const double* d_x0, const double* d_xref,
  * Algorithm 1's receding-horizon shift, the last element repeated).
  * After mppi_step, u0, the status word and the sequence are written by the
  * step itself into mapped pinned host memory, followed (after a system-scope
- * fence) by the step's iteration number.  The call then returns as soon
+ * fence) by the launch's number.  The call then returns as soon
  * as that number shows the last enqueued step, which can be before its
  * kernel has retired; the stream keeps the order of later work.  If the
  * stream ends without it (an error), when U is asked for after
- * mppi_set_state, or after mppi_step_device, it synchronises with the
+ * mppi_set_state, or after mppi_step_device or a step enqueued while its
+ * stream was being captured, it synchronises with the
  * context's last stream and copies what the mirror does not hold.  Errors: MPPI_ESTATE (no step has run),
  * MPPI_ETIMEOUT (a bounded device wait of the step expired), MPPI_ECUDA. */
 int mppi_get_control(mppi_ctx* c, double* u0, double* U);

@@ -378,7 +378,10 @@ struct mppi_ctx {
   bool stepped = false;
   bool mirrored = false;  // the last step writes the host mirror (mppi_step)
   bool mirror_U = false;  // and the sequence has not been set from the host since
-  uint64_t iter = 0;  // iteration counter of the device state after the steps enqueued so far
+  // Number of the last step that writes the mirror: one for each launch, never
+  // used twice.  (The device's iteration counter would not do: graphs that the
+  // caller captured move it on unseen, and mppi_set_state puts it back.)
+  uint32_t seq = 0;
 };
 
 namespace {
@@ -877,6 +880,7 @@ int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream,
   cudaStream_t s = stream ? (cudaStream_t)stream : c->own;
   if (const int rc = order_step(c, s)) return rc;
   if (mirror) {
+    c->D.seq = (int)++c->seq;
     c->fn<<<(c->D.nTiles + c->D.chunk - 1) / c->D.chunk, c->tl.threads, c->smem, s>>>(c->D, x0, xref);
   } else {
     CtrlDesc D = c->D;
@@ -888,7 +892,6 @@ int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream,
   c->order = nullptr;
   c->stepped = true;
   c->mirrored = c->mirror_U = mirror;
-  ++c->iter;
   return MPPI_OK;
 }
 }  // namespace
@@ -915,10 +918,12 @@ int mppi_step(mppi_ctx* c, const double* x0, const double* xref, void* stream) {
   } else {
     for (int t = 0; t <= T; ++t) memcpy(h + n + t * n, c->p.x_goal, sizeof(double) * n);
   }
-  const int rc = launch_step(c, c->h_in_dev[b], c->h_in_dev[b] + n, s, true);
+  // (a captured step has no number of its own: each replay would leave the same)
+  const bool live = !capturing(s);
+  const int rc = launch_step(c, c->h_in_dev[b], c->h_in_dev[b] + n, s, live);
   if (rc) return rc;
   CK(cudaEventRecord(c->in_ev[b], s));
-  if (!capturing(s)) c->order = c->in_ev[b];
+  if (live) c->order = c->in_ev[b];
   c->in_ev_pending[b] = true;
   c->in_next = b ^ 1;
   return MPPI_OK;
@@ -935,7 +940,7 @@ int mppi_get_control(mppi_ctx* c, double* u0, double* U) {
     // output, without waiting for the kernel to retire.  The stream is
     // polled now and then, so a step that ended without writing (an error)
     // falls through to the synchronisation below, which reports it.
-    const int want = (int)(uint32_t)c->iter;
+    const int want = (int)c->seq;
     volatile int* seq = &c->h_out->seq;
     for (unsigned n = 1;; ++n) {
       if (*seq == want) {
@@ -1049,9 +1054,7 @@ int mppi_set_state(mppi_ctx* c, const double* U, double S_e, double beta, int32_
   st.first = first ? 1 : 0;
   st.iter = iter;
   st.status = 0;
-  c->iter = iter;
   c->mirror_U = false;
-  c->h_out->seq = (int)(uint32_t)iter;  // not the next step's number, wherever the count was before
   CK(cudaMemcpy(c->d_U, U, sizeof(double) * 2 * c->p.T, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(c->d_st, &st, sizeof(DevState), cudaMemcpyHostToDevice));
   prep_kernel<<<1, 256, 0, c->own>>>(c->D, 0);

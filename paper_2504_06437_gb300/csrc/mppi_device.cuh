@@ -97,7 +97,7 @@ struct DevState {
 struct __align__(16) HostOut {
   double u0[2];  // u*_0
   int status;    // kStatus*
-  int seq;       // low 32 bits of the step's iteration counter + 1
+  int seq;       // the launch's number (CtrlDesc::seq)
 };
 
 // Everything a CTA needs to process one tile of one controller.
@@ -140,6 +140,7 @@ struct CtrlDesc {
   uint8_t* coll;             // K
   double* Ustar;             // T x 2
   HostOut* host_out;         // device alias of the host mirror, or null
+  int seq;                   // what the step leaves there when its outputs are in it
   double* ctl_out;           // the allocation-free step: where the caller keeps its state
   double* u0_out;            // and its control; null elsewhere
 };

@@ -572,7 +572,7 @@ __device__ __forceinline__ void final_stage(const CtrlDesc& D, char* smem, const
         D.host_out->u0[1] = us0[1];
         D.host_out->status = *reinterpret_cast<volatile int*>(&st->status);
         __threadfence_system();
-        *reinterpret_cast<volatile int*>(&D.host_out->seq) = (int)(uint32_t)(ts.iter + 1ull);
+        *reinterpret_cast<volatile int*>(&D.host_out->seq) = D.seq;
       }
       constexpr int n = Dyn<MODEL>::n;
       double xn[6] = {0, 0, 0, 0, 0, 0};
