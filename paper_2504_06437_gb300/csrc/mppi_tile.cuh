@@ -52,16 +52,31 @@ __device__ inline void sgf_weights(float* w, int W, int p, int tid, int nthreads
   }
 }
 
-// g^e for 0 <= e <= MPPI_MAX_T by repeated squaring: nine products in a row at
-// most, where pow takes several times as many FP64 operations; within e
-// roundings, far below the FP32 weights it goes into.
-__device__ __forceinline__ double pow_int(double g, int e) {
-  double r = 1.0;
-  for (; e; e >>= 1) {
-    if (e & 1) r *= g;
-    g *= g;
+// S_e = sum_{i<e} g^i = (1 - g^e) / (1 - g) and C_e = sum_{i=1..e} S_i for
+// 1 <= e <= MPPI_MAX_T, from the highest bit of e down: with p = g^m,
+//   S_2m = S_m (1 + p),  C_2m = C_m (1 + p) + m S_m,
+//   S_(m+1) = 1 + g S_m, C_(m+1) = C_m + S_(m+1).
+// Every term is positive, so both are right to a few roundings however close
+// g is to 1, where the quotients cancel: at g = 1 - 1e-8 and e = 256 the form
+// (e - g S_e) / (1 - g) of C_e is 2e-5 off with pow and 1e-3 off with g^e by
+// repeated squaring.  Some twenty FP64 operations in a row.
+__device__ __forceinline__ double geometric_sums(double g, int e, double* C_out) {
+  double p = g, S = 1.0, C = 1.0;  // m = 1
+  int m = 1;
+  for (int bit = 31 - __clz(e); --bit >= 0;) {
+    C = C * (1.0 + p) + m * S;
+    S *= 1.0 + p;
+    p *= p;
+    m *= 2;
+    if ((e >> bit) & 1) {
+      S = 1.0 + g * S;
+      C += S;
+      p *= g;
+      ++m;
+    }
   }
-  return r;
+  *C_out = C;
+  return S;
 }
 
 // Constants of the controller that never change: the unrolled DBaS weights
@@ -70,15 +85,14 @@ __device__ __forceinline__ double pow_int(double g, int e) {
 __device__ inline void init_constants(const CtrlDesc& D, int tid, int nthreads) {
   const int T = D.T;
   const double g = D.gamma_bas;
-  const double q = 1.0 / (1.0 - g);
+  double C;
   for (int t = tid; t < T; t += nthreads) {
     // step t produces x_{t+1}: c_{t+1} = (1 - g^(T - t)) / (1 - g)
-    D.cw[t] = (float)(D.R_B_d * ((1.0 - pow_int(g, T - t)) * q));
+    D.cw[t] = (float)(D.R_B_d * geometric_sums(g, T - t, &C));
   }
   if (tid == nthreads - 1) {
-    const double g1 = g * (1.0 - pow_int(g, T)) * q;
-    D.st->g1 = g1;
-    D.st->csum = (T - g1) * q;
+    D.st->g1 = g * geometric_sums(g, T, &C);
+    D.st->csum = C;
   }
   if (D.sgf_wp)
     sgf_weights(D.cw + sgf_table_offset(T), D.sgf_wp & 0xff, D.sgf_wp >> 8, tid, nthreads);
