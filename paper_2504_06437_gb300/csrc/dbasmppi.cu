@@ -1251,11 +1251,15 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   c.D.ctl_out = d_ctl;
   c.D.u0_out = d_u0;
   // a tile's bulk copy takes whole 16-byte units from a 16-byte boundary: an
-  // even number of obstacles that starts on one is read where it lies
+  // even number of obstacles that starts on one is read where it lies.  The
+  // prologue copies the others, by loads of 8 bytes; a set off that boundary
+  // takes a copy of its own
   const bool in_place = J > 0 && J % 2 == 0 && ((uintptr_t)d_obst & 15u) == 0;
+  const bool by_loads = J > 0 && !in_place && ((uintptr_t)d_obst & 7u) == 0;
   if (in_place) c.D.obst = d_obst;
-  static_prologue<<<1, 256, 0, s>>>(c.D, d_ctl, in_place || J == 0 ? nullptr : d_obst,
-                                    2 * (nGroups + 1));
+  if (J > 0 && !in_place && !by_loads)
+    CK(cudaMemcpyAsync(c.d_obst, d_obst, sizeof(double) * 3 * J, cudaMemcpyDeviceToDevice, s));
+  static_prologue<<<1, 256, 0, s>>>(c.D, d_ctl, by_loads ? d_obst : nullptr, 2 * (nGroups + 1));
   CK(cudaGetLastError());
   fn<<<(nTiles + chunk - 1) / chunk, c.tl.threads, c.smem, s>>>(c.D, d_x0, d_xref);
   CK(cudaGetLastError());

@@ -11,17 +11,20 @@ from paper_2504_06437_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-def _static(w, obstacles):
+def _static(w, obstacles, shift=0):
     import torch
     from paper_2504_06437_gb300 import binding
     lib = binding.load()
     p, T, x = w.params, int(w.params["T"]), w.x_start
     f64 = lambda a: torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")  # noqa: E731
-    d_o, d_x, d_r, d_U = f64(obstacles), f64(x), f64(w.reference(x)), f64(np.zeros((T, 2)))
+    # the set starts `shift` bytes off a boundary
+    d_o = torch.zeros(24 * len(obstacles) + 16, dtype=torch.uint8, device="cuda")
+    d_o[shift:shift + 24 * len(obstacles)] = f64(obstacles).view(torch.uint8).flatten()
+    d_x, d_r, d_U = f64(x), f64(w.reference(x)), f64(np.zeros((T, 2)))
     d_ctl, d_u0 = f64([p["mu_coarse"], 0.0, 1.0, 0.0, 0.0]), f64(np.zeros(2))
     d_c, params = f64(np.zeros(int(p["K"]))), binding.make_params(p)
     ptr = lambda a: C.c_void_p(a.data_ptr())  # noqa: E731
-    rc = lib.mppi_step_static(C.byref(params), ptr(d_o), C.c_int32(len(obstacles)), ptr(d_x), ptr(d_r), ptr(d_U),
+    rc = lib.mppi_step_static(C.byref(params), C.c_void_p(d_o.data_ptr() + shift), C.c_int32(len(obstacles)), ptr(d_x), ptr(d_r), ptr(d_U),
                               ptr(d_ctl), ptr(d_u0), ptr(d_c), C.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert rc == 0, lib.mppi_last_error().decode()
     torch.cuda.synchronize()
@@ -62,3 +65,14 @@ def test_an_obstacle_out_of_sight_adds_nothing(where):
     a, b = _static(w, w.obstacles), _static(w, pad)
     assert np.isfinite(b[0]).all()
     assert (np.abs(a[0] - b[0]) <= 2e-5 * np.maximum(np.abs(a[0]), 1.0)).all()
+
+
+@pytest.mark.parametrize("J", [1, 60, 61])
+@pytest.mark.parametrize("shift", [1, 4, 8])
+def test_a_set_off_every_boundary_is_copied(J, shift):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    w = _world("quad2d", J)
+    for a, b in zip(_static(w, w.obstacles), _static(w, w.obstacles, shift)):
+        assert np.array_equal(a, b)
