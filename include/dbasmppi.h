@@ -314,9 +314,9 @@ int mppi_debug_wait_probe(int64_t max_cycles, int32_t arrive);
  * call returns without waiting.  Set-up happens on first use, not at load:
  * the first call on each device looks up the array's device address (once,
  * under a lock, so host threads may race to it), and the first call for each
- * (device, model, smoothing on or off) sets that step kernel's shared-memory
- * limit and queries its occupancy; a new launch shape queries occupancy
- * again.  Make one such call for every (device, model, smoothing) you will
+ * (device, model, smoothing on or off) sets the shared-memory limit of those
+ * step kernels, the ones for many obstacles among them, and queries occupancy;
+ * a new launch shape queries occupancy again.  Make one such call for every (device, model, smoothing) you will
  * use before any stream capture.  Every call shares the one array: calls
  * whose GPU work overlaps (other streams, other host threads) race; order
  * them.  Errors:

@@ -264,65 +264,80 @@ int max_smem_optin() {
 }
 
 // Step kernel of a launch: the 96-register form, or the 80-register form
-// (_r80) when the grid spans more than one wave of the 96-register form and
-// the lower cap raises the CTAs resident per SM.  The shared-memory limit
+// when it fits more CTAs per SM and the grid spans more than one wave of
+// the other (at create and on set_obstacles).  The dynamic shared-memory limit
 // of a model's step kernels is raised once per device; the last decision per
-// device is kept, so a repeated configuration costs no occupancy query
-// (the allocation-free entry point calls this every step).
+// device and form is kept, so a repeated configuration costs no occupancy
+// query (the allocation-free entry point calls this every step).  The forms
+// beyond the plain one need a query only for the chunk, and only where the
+// grid could hold more than one tile per CTA.
 struct PickMemo {
   int model, npos, threads, smem, nTiles, chunk;
   bool far;
   StepFn fn;
 };
 std::mutex g_pick_mu;
-bool g_step_attr[kMaxPickDevices][MPPI_NUM_MODELS][2] = {};
-bool g_form_attr[kMaxPickDevices][2][MPPI_NUM_MODELS][2] = {};
-PickMemo g_pick_memo[kMaxPickDevices] = {};
+bool g_step_attr[kMaxPickDevices][3][MPPI_NUM_MODELS][2] = {};  // [form] .. [far-field cells]
+PickMemo g_pick_memo[kMaxPickDevices][3] = {};
 
+// Only one model's kernels of one form, with or without cells: with lazy
+// module loading, touching a kernel loads its module, and what a process
+// never steps stays unloaded.
+int prepare_step_kernels(int dev, int form, int model, bool far) {
+  bool& done = g_step_attr[dev][form][model][far ? 1 : 0];
+  if (done) return MPPI_OK;
+  const int lim = max_smem_optin();
+  for (int np : {8, 14}) {
+    if (form != kFormPlain) {
+      CK(cudaFuncSetAttribute(pick_form_kernel(form, model, np, far),
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    } else {
+      for (bool r80 : {false, true})
+        CK(cudaFuncSetAttribute(pick_kernel(model, np, r80, far),
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    }
+  }
+  done = true;
+  return MPPI_OK;
+}
+
+// both: the kernels of the other choice of `far` are prepared as well, so that
+// a later call with more or fewer obstacles finds them ready.
 int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, int form, bool far,
-                       StepFn* out, int* chunk) {
+                       StepFn* out, int* chunk, bool both = false) {
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxPickDevices) return fail(MPPI_EINVAL, "device %d out of range", dev);
   std::lock_guard<std::mutex> lock(g_pick_mu);
-  if (form != kFormPlain) {
-    bool& done = g_form_attr[dev][form == kFormGrid ? 1 : 0][model][far ? 1 : 0];
-    if (!done) {
-      const int lim = max_smem_optin();
-      for (int np : {8, 14})
-        CK(cudaFuncSetAttribute(pick_form_kernel(form, model, np, far),
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-      done = true;
-    }
+  if (const int rc = prepare_step_kernels(dev, form, model, far)) return rc;
+  if (both)
+    if (const int rc = prepare_step_kernels(dev, form, model, !far)) return rc;
+  if (form != kFormPlain && chunk_of(nTiles, num_sms()) == 1) {
     *out = pick_form_kernel(form, model, npos, far);
-    int occ = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, *out, threads, smem));
-    *chunk = chunk_of(nTiles, (long)std::max(occ, 1) * num_sms());
+    *chunk = 1;
     return MPPI_OK;
   }
-  // only this model's kernels: with lazy module loading, touching a kernel
-  // loads its module, and the models a process never steps stay unloaded
-  if (!g_step_attr[dev][model][far ? 1 : 0]) {
-    const int lim = max_smem_optin();
-    for (int np : {8, 14})
-      for (bool r80 : {false, true})
-        CK(cudaFuncSetAttribute(pick_kernel(model, np, r80, far),
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    g_step_attr[dev][model][far ? 1 : 0] = true;
-  }
-  PickMemo& m = g_pick_memo[dev];
-  if (m.fn && m.far == far && m.model == model && m.npos == npos && m.threads == threads && m.smem == smem &&
-      m.nTiles == nTiles) {
+  PickMemo& m = g_pick_memo[dev][form];
+  if (m.fn && m.far == far && m.model == model && m.npos == npos && m.threads == threads &&
+      m.smem == smem && m.nTiles == nTiles) {
     *out = m.fn;
     *chunk = m.chunk;
     return MPPI_OK;
   }
-  const StepFn hi = pick_kernel(model, npos, false, far), lo = pick_kernel(model, npos, true, far);
-  int occ_hi = 0, occ_lo = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_hi, hi, threads, smem));
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_lo, lo, threads, smem));
-  const StepFn fn = (occ_lo > occ_hi && (long)nTiles > (long)occ_hi * num_sms()) ? lo : hi;
-  *chunk = chunk_of(nTiles, (long)std::max(fn == lo ? occ_lo : occ_hi, 1) * num_sms());
+  StepFn fn = form == kFormPlain ? pick_kernel(model, npos, false, far)
+                                 : pick_form_kernel(form, model, npos, far);
+  int occ = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
+  if (form == kFormPlain) {
+    const StepFn lo = pick_kernel(model, npos, true, far);
+    int occ_lo = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_lo, lo, threads, smem));
+    if (occ_lo > occ && (long)nTiles > (long)occ * num_sms()) {
+      fn = lo;
+      occ = occ_lo;
+    }
+  }
+  *chunk = chunk_of(nTiles, (long)std::max(occ, 1) * num_sms());
   m = PickMemo{model, npos, threads, smem, nTiles, *chunk, far, fn};
   *out = fn;
   return MPPI_OK;
@@ -1227,7 +1242,8 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   StepFn fn = nullptr;  // picked before anything is launched
   int chunk = 1;
   rc = choose_step_kernel(p->model, c.tl.positions_per_thread, c.tl.threads, c.smem, nTiles,
-                          p->sgf_window > 0 ? kFormSgf : kFormPlain, c.nc > 0, &fn, &chunk);
+                          p->sgf_window > 0 ? kFormSgf : kFormPlain, c.nc > 0, &fn, &chunk,
+                          /*both=*/true);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   c.d_U = d_U;
