@@ -292,6 +292,14 @@ int mppi_debug_draws(const mppi_params* p, double S_e, uint64_t iter, int32_t K,
  * The paper has no counterpart; this is test support for the failure path. */
 int mppi_debug_wait_probe(int64_t max_cycles, int32_t arrive);
 
+/* Diagnostic: the form of the following steps of a context.  cells 1 = the
+ * library's choice, 0 = every pair of shape point and obstacle one by one, no
+ * far-field cells; tiles_per_cta = tiles that a CTA takes in a row (1, 2, 4
+ * or 8), 0 = the library's choice.  The number in a row changes no result; cells
+ * change costs by rounding.  For tests that compare the forms; the paper has
+ * no counterpart.  Errors: MPPI_ESTATE (NULL context), MPPI_EINVAL. */
+int mppi_debug_set_form(mppi_ctx* c, int32_t cells, int32_t tiles_per_cta);
+
 /* One step without any device allocation and without a context, for callers
  * that may not allocate once they run: real-time control loops that keep
  * every step's latency bounded (cudaMalloc can block and synchronise the

@@ -151,6 +151,7 @@ def load():
     lib.mppi_debug_draws.argtypes = [C.POINTER(Params), C.c_double, C.c_uint64, C.c_int32,
                                      C.c_int32, C.POINTER(C.c_uint32), C.POINTER(C.c_float)]
     lib.mppi_debug_wait_probe.argtypes = [C.c_int64, C.c_int32]
+    lib.mppi_debug_set_form.argtypes = [vp, C.c_int32, C.c_int32]
     lib.mppi_autotune_grid.argtypes = [C.POINTER(Params), _dp, C.c_int32, C.POINTER(C.c_float),
                                        C.c_int32, C.c_int32, C.c_double, C.c_double, C.c_double,
                                        C.c_int32, C.POINTER(Tiling), C.POINTER(C.c_float)]
@@ -377,6 +378,10 @@ class Controller:
         r = C.c_int32()
         _check(load().mppi_get_kernel_regs(self.h, C.byref(r)))
         return r.value
+
+    def debug_set_form(self, cells: bool = True, tiles_per_cta: int = 0):
+        """Fix the form of the following steps (mppi_debug_set_form)."""
+        _check(load().mppi_debug_set_form(self.h, int(bool(cells)), int(tiles_per_cta)))
 
     def io_bytes(self):
         a, b = C.c_uint64(), C.c_uint64()

@@ -354,6 +354,8 @@ struct mppi_ctx {
   int Jcap = 0;
   int smem = 0;
   int nc = 0;  // far-field cells of a tile
+  bool cells = true;  // false: every obstacle directly (mppi_debug_set_form)
+  int row = 0;        // tiles of a CTA, 0 = the library's choice (mppi_debug_set_form)
   CtrlDesc D;
   StepFn fn = nullptr;
   double* d_U = nullptr;
@@ -477,7 +479,7 @@ void default_shape(int K, int sms, int* S, int* threads) {
 }
 
 int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tiling* out,
-                  int* smem_out, int* nc_out, bool batched = false) {
+                  int* smem_out, int* nc_out, bool batched = false, bool cells = true) {
   const int sms = num_sms();
   const int n = state_dim(p->model);
   mppi_tiling t = {0, 0, 0, 0};
@@ -515,6 +517,7 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
     // whose rows are wider and whose serving form has 13 KB of its own: a
     // controller takes them alone, batched and served or not at all
     int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads);
+    if (!cells) nc = 0;
     if (nc > 0 && smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, nc,
                               true).total > limit - kServeStatic)
       nc = 0;
@@ -755,7 +758,7 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   }
   mppi_tiling t;
   int smem = 0, nc = 0;
-  int rc = choose_tiling(&c->p, &c->tl, J, &t, &smem, &nc);
+  int rc = choose_tiling(&c->p, &c->tl, J, &t, &smem, &nc, false, c->cells);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->last));
   const size_t bytes = (size_t)align_up(24 * (J > 0 ? J : 1), 16);
@@ -786,7 +789,7 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   c->fn = fn;
   c->D.J = J;
   c->D.nc = nc;
-  c->D.chunk = chunk;
+  c->D.chunk = c->row ? c->row : chunk;
   c->D.obst = c->d_obst;
   return MPPI_OK;
 }
@@ -852,7 +855,30 @@ int mppi_set_grid(mppi_ctx* c, const float* sdf, int32_t nx, int32_t ny, double 
   cudaFree(c->d_grid);
   c->d_grid = nb;
   c->fn = fn;
-  c->D.chunk = chunk;
+  c->D.chunk = c->row ? c->row : chunk;
+  return MPPI_OK;
+}
+
+int mppi_debug_set_form(mppi_ctx* c, int32_t cells, int32_t tiles_per_cta) {
+  if (!c) return fail(MPPI_ESTATE, "context is NULL");
+  if (cells < 0 || cells > 1) return fail(MPPI_EINVAL, "cells must be 0 or 1");
+  // powers of two up to kMaxChunk, of which merge groups hold whole numbers
+  if (tiles_per_cta < 0 || tiles_per_cta > kMaxChunk || (tiles_per_cta & (tiles_per_cta - 1)))
+    return fail(MPPI_EINVAL, "tiles_per_cta must be 0, 1, 2, 4 or 8");
+  mppi_tiling t;
+  int smem = 0, nc = 0, chunk = 1;
+  int rc = choose_tiling(&c->p, &c->tl, c->D.J, &t, &smem, &nc, false, cells != 0);
+  if (rc) return rc;
+  StepFn fn = nullptr;
+  rc = choose_step_kernel(c->p.model, t.positions_per_thread, t.threads, smem, c->D.nTiles,
+                          step_form(c), nc > 0, &fn, &chunk);
+  if (rc) return rc;
+  c->cells = cells != 0;
+  c->row = tiles_per_cta;
+  c->smem = smem;
+  c->nc = c->D.nc = nc;
+  c->fn = fn;
+  c->D.chunk = c->row ? c->row : chunk;
   return MPPI_OK;
 }
 

@@ -497,14 +497,14 @@ struct Dyn {
 };
 
 // ------------------------------------------------------------ tile kernel body
-// Weights of at least 1 / kRefShare are settled by direct sums
-// (refine_samples): at most kRefShare samples can have one.  Over two steps of
-// 84 problems U* then stays within 1e-5 of the direct evaluation's but for
-// three whose weights hang on the last bit of a cost; with 32 the first step's
-// largest differences are ten times those with 512, for 3 us less.
+// Samples with a weight of at least 1 / kRefShare are summed directly once
+// more (refine_samples); at most kRefShare samples can have one (their weights
+// add up to 1 at most; the last roundings of 128 weights of 1 / 128 each can
+// not make room for another).  Their numbers and the changes of their costs
+// lie in the reduction scratch.
 constexpr int kRefShare = 128;
-constexpr int kRefMax = kRefShare + 8;
-static_assert(4 * kRefMax <= 8 * 4 * 32, "the list lies in the reduction scratch");
+constexpr int kRefMax = kRefShare;
+static_assert(8 * kRefMax <= 8 * 4 * 32, "the list lies in the reduction scratch");
 struct TileScratch {
   uint64_t mbar;
   int flag;

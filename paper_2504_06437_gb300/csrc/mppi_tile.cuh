@@ -616,8 +616,8 @@ __device__ __forceinline__ void final_stage(const CtrlDesc& D, char* smem, const
   }
 }
 
-// The samples that hold at least 1 / kRefShare of the normaliser Z, at most
-// kRefShare of them: into ref_k, ascending.  Called by the last CTA after
+// The samples that hold at least 1 / kRefShare of the normaliser Z: into
+// ref_k, ascending (none, should there be more than kRefMax).  Called by the last CTA after
 // the last merge, whose source scales (the tiles', or with two levels the
 // groups') scl holds; the tiles' minima and then the costs of the few tiles
 // that can hold one are read again.  Scratch: ref_tile (kRefMax ints).
@@ -639,7 +639,7 @@ __device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, 
   }
   __syncthreads();
   const double base = ts.base, ref = (double)ts.ref;
-  const int n_tile = min(ts.n_tile, kRefMax);
+  const int n_tile = ts.n_tile <= kRefMax ? ts.n_tile : 0;
   for (int q = tid >> 5; q < n_tile; q += nthreads >> 5) {
     const int k = ref_tile[q] * D.S + lane;
     if (lane < D.S && k < D.K) {
@@ -652,7 +652,7 @@ __device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, 
   }
   __syncthreads();
   // in ascending order: the sums do not depend on who came first
-  const int n = min(ts.n_ref, kRefMax);
+  const int n = ts.n_ref <= kRefMax ? ts.n_ref : 0;
   int v[kRefPer], r[kRefPer];
 #pragma unroll
   for (int q = 0; q < kRefPer; ++q) {
@@ -670,19 +670,44 @@ __device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, 
   __syncthreads();
 }
 
+// The clamped controls of the listed samples r0 .. r0 + Sc - 1, drawn anew
+// (the generator is counter based), at V[t Sc + s].
+__device__ __forceinline__ void refine_draws(const CtrlDesc& D, const TileScratch& ts,
+                                             const int* ref_k, const float2* Uf, float2* V, int r0,
+                                             int Sc, int tid, int nthreads) {
+  const DevState* st = D.st;
+  const uint32_t it_lo = (uint32_t)(ts.iter & 0xffffffffull), it_hi = (uint32_t)(ts.iter >> 32);
+  for (int i = tid; i < D.T * Sc; i += nthreads) {
+    const int t = i / Sc, s = i - t * Sc;
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)ref_k[r0 + s], (uint32_t)t, it_lo, it_hi),
+                                  D.key0, D.key1);
+    const float2 du = nln_draw(r, st->L00, st->L10, st->L11, D.ln_mu, D.ln_sigma), u = Uf[t];
+    V[i] = make_float2(fminf(fmaxf(u.x + du.x, D.umin[0]), D.umax[0]),
+                       fminf(fmaxf(u.y + du.y, D.umin[1]), D.umax[1]));
+  }
+}
+
 // Second look at the samples that carry the weights, after the last merge of
-// a step whose tiles used far-field cells: their costs once more with every
-// obstacle summed directly, and the change of their weights put into Z and
-// the merged column sums.  A weight is the exponential of a cost difference,
-// so where a few samples share all of it the rounding of their costs goes
-// straight into U*: some 1e-5 of a barrier cost of hundreds, whichever way it
-// is summed.  Taking those few again leaves the polynomial no say in it: they
-// end with the bits of the direct evaluation.  They are drawn and rolled out
-// anew (the generator is counter based).  The last CTA runs this alone, a
-// chain of latencies (list 2.5, draws 1, rollout 2, barrier 2 to 20, costs 1,
-// columns 1 us); out of line, so that its registers leave the tile's code as
-// it is: as a second round of the tile's own code it took the batch kernel
-// from 13.4 to 14.4 ms.
+// a step whose tiles used far-field cells.  A weight is the exponential of a
+// cost difference, so where a few samples share all of it the rounding of
+// their costs goes straight into U*: some 1e-5 of a barrier cost of hundreds,
+// whichever way it is summed.  The costs of those few are formed once more
+// with every obstacle summed directly, so that U* hangs on the roundings of
+// the direct evaluation and not on how poses were cut into cells (the cells'
+// sums are no less exact).
+// What the two sums of a sample differ by has a part that all samples share,
+// for instance where a term of 1 / h_eps is paired with another obstacle.
+// Only the listed samples are summed again, so that part would shift their
+// weights against all the others'.  It is taken out: with m the mean of the
+// differences delta, weighted by the weights, a listed sample's cost changes by
+// delta - m.  Z then never falls (exp is convex: the mean of
+// exp(-(delta - m) / lambda) is at least 1), so it stays at least 1, as the
+// final stage assumes.  Where the differences left over exceed lambda the
+// costs' rounding decides the weights in either sum, and the first one stays.
+// The last CTA runs this alone, a chain of latencies (list 2.5, draws 1,
+// rollout 2, barrier 2 to 20, costs 1, columns 1 us); out of line, so that its
+// registers leave the tile's code as it is: as a second round of the tile's
+// own code it took the batch kernel from 13.4 to 14.4 ms.
 template <int MODEL, int NPOS, bool BATCHED, bool GRID>
 __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const CtrlDesc& D = BATCHED ? tile_desc() : D_;
@@ -693,31 +718,23 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const int T = D.T, P = D.P, J = D.J;
   const SmemLayout L = smem_layout(T, D.S, P, J, Dyn<MODEL>::n, D.nscl, nwarps, D.nc, BATCHED);
   int* ref_k = reinterpret_cast<int*>(smem + L.red);
+  float* delta = reinterpret_cast<float*>(smem + L.red) + kRefMax;
   refine_list(D, ts, reinterpret_cast<const float*>(smem + L.scl), ref_k,
               reinterpret_cast<int*>(smem + L.region), tid, nthreads);
   const float2* Uf = reinterpret_cast<const float2*>(smem + L.Uf);
   const float* cw = reinterpret_cast<const float*>(smem + L.cw);
-  float* eS = reinterpret_cast<float*>(smem + L.eS);
   float* scH = reinterpret_cast<float*>(smem + L.scH);
   float* scL = reinterpret_cast<float*>(smem + L.scL);
   float* col_hi = reinterpret_cast<float*>(smem + L.colhi);
   float* col_lo = reinterpret_cast<float*>(smem + L.collo);
   float4* pose = reinterpret_cast<float4*>(smem + L.region);
   const float2* uB = reinterpret_cast<const float2*>(pose);
-  const DevState* st = D.st;
-  const uint32_t it_lo = (uint32_t)(ts.iter & 0xffffffffull), it_hi = (uint32_t)(ts.iter >> 32);
   const int n_ref = ts.n_ref;
+  if (n_ref == 0) return;
   for (int r0 = 0; r0 < n_ref; r0 += D.S) {
     const int Sc = min(D.S, n_ref - r0);
     float2* V = reinterpret_cast<float2*>(pose + T * Sc);
-    for (int i = tid; i < T * Sc; i += nthreads) {
-      const int t = i / Sc, s = i - t * Sc;
-      const uint4 r = philox4x32_10(make_uint4((uint32_t)ref_k[r0 + s], (uint32_t)t, it_lo, it_hi),
-                                    D.key0, D.key1);
-      const float2 du = nln_draw(r, st->L00, st->L10, st->L11, D.ln_mu, D.ln_sigma), u = Uf[t];
-      V[i] = make_float2(fminf(fmaxf(u.x + du.x, D.umin[0]), D.umax[0]),
-                         fminf(fmaxf(u.y + du.y, D.umin[1]), D.umax[1]));
-    }
+    refine_draws(D, ts, ref_k, Uf, V, r0, Sc, tid, nthreads);
     __syncthreads();
     const float* xi = reinterpret_cast<const float*>(smem + L.xi);
     float sin0, cos0;
@@ -741,8 +758,6 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
                                GRID ? &grid_shared() : nullptr);
     __syncthreads();
     for (int s = warp; s < Sc; s += nwarps) {
-      const int k = ref_k[r0 + s];
-      const double was = __ldcg(D.costs + k) - ts.base;
       FF b = {0.0f, 0.0f};
       for (int t = lane; t < T; t += 32) {
         const float2 v = uB[2 * (t * Sc + s)];
@@ -753,25 +768,66 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
       b = warp_sum_ff(b);
       if (lane == 0) {
         const FF c = ff_norm(ff_sum(FF{scH[s], scL[s]}, b));
-        const double now = (double)c.hi + (double)c.lo;
-        D.costs[k] = ts.base + now;
-        eS[s] = expf(-(float)(now - (double)ts.ref) * D.inv_lambda_f) -
-                expf(-(float)(was - (double)ts.ref) * D.inv_lambda_f);
+        const double was = __ldcg(D.costs + ref_k[r0 + s]) - ts.base;
+        delta[r0 + s] = (float)((double)c.hi + (double)c.lo - was);
       }
     }
     __syncthreads();
+  }
+  if (warp == 0) {
+    constexpr int kPer = kRefMax / 32;
+    double was[kPer];
+    float e[kPer];
+    float se = 0.0f, sd = 0.0f;
+    bool near = true;  // (false for a difference that is no number)
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = lane + 32 * q;
+      was[q] = i < n_ref ? __ldcg(D.costs + ref_k[i]) - ts.base : 0.0;
+      e[q] = i < n_ref ? expf(-(float)(was[q] - (double)ts.ref) * D.inv_lambda_f) : 0.0f;
+      se += e[q];
+      if (i < n_ref) sd = fmaf(e[q], delta[i], sd);
+    }
+    const float m = warp_sum_f(sd) / warp_sum_f(se);  // the same in every lane
+#pragma unroll
+    for (int q = 0; q < kPer; ++q)
+      if (lane + 32 * q < n_ref)
+        near = near && fabsf(delta[lane + 32 * q] - m) * D.inv_lambda_f <= 1.0f;
+    const bool take = __all_sync(0xffffffffu, near);
+    FF z = {0.0f, 0.0f};
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = lane + 32 * q;
+      if (take && i < n_ref) {
+        const double now = was[q] + (double)(delta[i] - m);
+        D.costs[ref_k[i]] = ts.base + now;
+        delta[i] = expf(-(float)(now - (double)ts.ref) * D.inv_lambda_f) - e[q];
+        ff_add(z, delta[i]);
+      }
+    }
+    __syncwarp();
+    z = warp_sum_ff(z);
+    if (lane == 0) {
+      ts.flag = take ? 1 : 0;
+      if (take) ts.Z = ff_norm(ff_sum(ts.Z, z));
+    }
+  }
+  __syncthreads();
+  if (!ts.flag) return;
+  for (int r0 = 0; r0 < n_ref; r0 += D.S) {
+    const int Sc = min(D.S, n_ref - r0);
+    float2* V = reinterpret_cast<float2*>(pose + T * Sc);
+    if (n_ref > D.S) {  // (else the only draws are still there)
+      refine_draws(D, ts, ref_k, Uf, V, r0, Sc, tid, nthreads);
+      __syncthreads();
+    }
     for (int c = tid; c < 2 * T; c += nthreads) {
       const float* Vt = reinterpret_cast<const float*>(V + (c >> 1) * Sc) + (c & 1);
       const float u = reinterpret_cast<const float*>(Uf)[c];
       FF a = {col_hi[c], col_lo[c]};
-      for (int s = 0; s < Sc; ++s) ff_add(a, eS[s] * (Vt[2 * s] - u));
+      for (int s = 0; s < Sc; ++s) ff_add(a, delta[r0 + s] * (Vt[2 * s] - u));
       col_hi[c] = a.hi;
       col_lo[c] = a.lo;
-    }
-    if (tid == 0) {
-      FF z = ts.Z;
-      for (int s = 0; s < Sc; ++s) ff_add(z, eS[s]);
-      ts.Z = ff_norm(z);
     }
     __syncthreads();
   }
