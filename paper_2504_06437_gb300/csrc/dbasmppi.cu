@@ -539,6 +539,14 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
   return MPPI_OK;
 }
 
+// The obstacle count and the cells that go with it.
+void set_cells(CtrlDesc& D, int J, int nc) {
+  D.J = J;
+  D.nc = nc;
+  D.look_max = 0.5f * (float)D.K / (float)num_sms();
+  D.look_over = nc > 0 ? (17.0f + far_setup_ops(nc, J, D.T * D.S * D.P)) / (float)J : 0.0f;
+}
+
 // Fill the descriptor from the parameters and the device buffers.
 void fill_desc(mppi_ctx* c) {
   const mppi_params* p = &c->p;
@@ -552,7 +560,6 @@ void fill_desc(mppi_ctx* c) {
   D.n = c->n;
   D.S = c->tl.samples_per_cta;
   D.NPOS = c->tl.positions_per_thread;
-  D.nc = c->nc;
   D.chunk = 1;
   D.nTiles = (p->K + D.S - 1) / D.S;
   D.GT = group_size(D.nTiles);
@@ -787,8 +794,7 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   c->smem = smem;
   c->nc = nc;
   c->fn = fn;
-  c->D.J = J;
-  c->D.nc = nc;
+  set_cells(c->D, J, nc);
   c->D.chunk = c->row ? c->row : chunk;
   c->D.obst = c->d_obst;
   return MPPI_OK;
@@ -876,7 +882,8 @@ int mppi_debug_set_form(mppi_ctx* c, int32_t cells, int32_t tiles_per_cta) {
   c->cells = cells != 0;
   c->row = tiles_per_cta;
   c->smem = smem;
-  c->nc = c->D.nc = nc;
+  c->nc = nc;
+  set_cells(c->D, c->D.J, nc);
   c->fn = fn;
   c->D.chunk = c->row ? c->row : chunk;
   return MPPI_OK;
@@ -1189,6 +1196,7 @@ __global__ void static_prologue(const __grid_constant__ CtrlDesc D, const double
     D.st->first = ctl[2] != 0.0 ? 1 : 0;
     D.st->iter = (unsigned long long)ctl[3];
     D.st->status = 0;
+    D.st->near = 0u;
   }
   for (int i = threadIdx.x; i < n_counters; i += blockDim.x) D.counters[i] = 0u;
   if (obst)
@@ -1288,7 +1296,7 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   c.d_coll = (uint8_t*)(base + o_coll);
   c.d_Ustar = (double*)(base + o_Ustar);
   fill_desc(&c);
-  c.D.J = J;
+  set_cells(c.D, J, c.nc);
   c.D.chunk = chunk;
   c.D.ctl_out = d_ctl;
   c.D.u0_out = d_u0;
@@ -1676,7 +1684,7 @@ int batch_write_desc(mppi_batch* b, int slot) {
   c.nc = s.nc;
   slot_layout(b, s, &c);
   fill_desc(&c);
-  c.D.J = s.J;
+  set_cells(c.D, s.J, s.nc);
   s.D = c.D;
   CK(cudaMemcpy(b->d_descs + slot, &s.D, sizeof(CtrlDesc), cudaMemcpyHostToDevice));
   return MPPI_OK;

@@ -73,7 +73,8 @@ struct DevState {
   double x1[6];      // last step: state after applying u*_0 (model prediction)
   double C0;         // sum_t gamma u_t^T (S_e Sigma)^-1 u_t of the next step
   double csum, g1;   // DBaS unrolling constants (see above)
-  float L00, L10, L11, pad;  // chol(S_e Sigma) of the next step
+  float L00, L10, L11;  // chol(S_e Sigma) of the next step
+  unsigned near;     // near obstacles of the tiles' cells (far_share); zero between steps
   unsigned long long iter;  // Philox counter words 2..3
   int first;         // 1 until the first step
   int status;        // kStatus*
@@ -107,6 +108,7 @@ struct CtrlDesc {
   int chunk;                 // tiles of a CTA of the one-controller kernels
   int nc;                    // far-field cells of a tile (far_cells), 0 = every pair directly
   float r_body;              // largest distance of a shape point from the body's position
+  float look_max, look_over; // bounds of the second look (look_samples)
   float dt, h_eps, C_coll, ln_mu, ln_sigma;
   float umin[2], umax[2];
   float Q[kMaxN], Qf[kMaxN];
@@ -224,6 +226,9 @@ __host__ __device__ inline int far_list_cap(int J) {
 // K 8192, T 40, J 60 (7e7) 104 us without, 86 to 92 us with them.
 constexpr int kFarCellPoints = 1024;
 constexpr float kFarMinSaved = 4.0e7f;
+__host__ __device__ inline float far_setup_ops(int nc, int J, int pts) {
+  return nc * (2800.0f + 53.0f * J) / pts;
+}
 __host__ __device__ inline int far_cells(int K, int T, int S, int P, int J, int npos,
                                          int nthreads) {
   const int gsz = 32 * (npos / P);
@@ -234,8 +239,7 @@ __host__ __device__ inline int far_cells(int K, int T, int S, int P, int J, int 
   if (nc > nthreads / 32) nc = nthreads / 32;
   if (nc > groups) nc = groups;
   if (nc < 1) nc = 1;
-  const float setup = nc * (2800.0f + 53.0f * J) / pts;
-  return (float)K * T * P * (0.9f * J - 17.0f - setup) >= kFarMinSaved ? nc : 0;
+  return (float)K * T * P * (0.9f * J - 17.0f - far_setup_ops(nc, J, pts)) >= kFarMinSaved ? nc : 0;
 }
 
 // Row stride of the tile's (step, sample) arrays (poses, clamped controls,

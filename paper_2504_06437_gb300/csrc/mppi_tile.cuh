@@ -670,6 +670,34 @@ __device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, 
   __syncthreads();
 }
 
+// A tile's share of near obstacles, in 256ths of its cells' obstacles, added to
+// the step's word.  Called by one warp, the cells set up.
+__device__ __forceinline__ void far_share(const CtrlDesc& D, const FarCell* cells, int nc, int lane) {
+  const int nn = lane < nc ? cells[lane].n_near : 0;
+  const unsigned near = __reduce_add_sync(0xffffffffu, (unsigned)(nn < 0 ? D.J : nn));
+  if (lane == 0) atomicAdd(&D.st->near, 256u * near / (unsigned)(nc * D.J));
+}
+
+// How many samples the second look may take.  One CTA sums them alone, n of
+// them in about n sms / K of the time that the direct evaluation of the whole
+// step takes, of which the cells saved the far obstacles' share less the
+// polynomials' and their set-up's (far_cells; look_over): at most half of what
+// was saved is given back.  Without a bound, at high temperatures, a vehicle at
+// K 221, T 132, J 378 took 654 us a step against 113 us without cells, one at
+// K 1076, T 156, J 577 913 us against 310 us.
+// None where every cell took its obstacles directly, where the direct sums are
+// the same bits; none where one sample has all the weight but 1 / kRefShare
+// or none can have that much; and none where the costs, and with them their
+// rounding, are small beside the temperature: at 4 lambda a rounding of the
+// cost moves a weight by 2^-22 of itself, as the exponential's own does.
+__device__ __forceinline__ int look_samples(const CtrlDesc& D, const TileScratch& ts,
+                                            unsigned share) {
+  if (!(ts.Z.hi > 1.0f + 1.0f / kRefShare) || ts.Z.hi > (float)kRefShare) return 0;
+  if (ts.ref * D.inv_lambda_f <= 4.0f) return 0;
+  const float near = (float)share / (256.0f * (float)D.nTiles);
+  return (int)fminf(D.look_max * (1.0f - near - D.look_over), (float)kRefMax);
+}
+
 // The clamped controls of the listed samples r0 .. r0 + Sc - 1, drawn anew
 // (the generator is counter based), at V[t Sc + s].
 __device__ __forceinline__ void refine_draws(const CtrlDesc& D, const TileScratch& ts,
@@ -716,6 +744,11 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const int tid = threadIdx.x, nthreads = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
   const int T = D.T, P = D.P, J = D.J;
+  unsigned* word = &D.st->near;
+  const int n_max = look_samples(D, ts, __ldcg(word));
+  __syncthreads();
+  if (tid == 0) *word = 0u;  // for the next step
+  if (n_max <= 0) return;
   const SmemLayout L = smem_layout(T, D.S, P, J, Dyn<MODEL>::n, D.nscl, nwarps, D.nc, BATCHED);
   int* ref_k = reinterpret_cast<int*>(smem + L.red);
   float* delta = reinterpret_cast<float*>(smem + L.red) + kRefMax;
@@ -730,7 +763,7 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   float4* pose = reinterpret_cast<float4*>(smem + L.region);
   const float2* uB = reinterpret_cast<const float2*>(pose);
   const int n_ref = ts.n_ref;
-  if (n_ref == 0) return;
+  if (n_ref == 0 || n_ref > n_max) return;
   for (int r0 = 0; r0 < n_ref; r0 += D.S) {
     const int Sc = min(D.S, n_ref - r0);
     float2* V = reinterpret_cast<float2*>(pose + T * Sc);
@@ -1110,6 +1143,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
                            lane);
       }
       __syncthreads();
+      if (warp == nwarps - 1) far_share(D, cells, nc, lane);
     }
   }
 
@@ -1270,10 +1304,8 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
                              D.inv_lambda_f, scl, zi, mbuf, &ts.ref, &ts.Z, col_hi, col_lo, tid,
                              nthreads);
   }
-  // (one sample with all but 1 / kRefShare of the weight needs no second look)
   if constexpr (FAR) {
-    if (D.nc > 0 && ts.Z.hi > 1.0f + 1.0f / kRefShare)
-      refine_samples<MODEL, NPOS, BATCHED, GRID>(D);
+    if (D.nc > 0) refine_samples<MODEL, NPOS, BATCHED, GRID>(D);
   }
   if constexpr (SGF) {
     if (D.sgf_wp)
