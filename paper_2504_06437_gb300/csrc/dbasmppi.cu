@@ -452,29 +452,40 @@ void free_ctx(mppi_ctx* c) {
 //    tile's chain of phases and the merge of its rows, so the fewest rows (one
 //    merge level) and the most warps win (quadrotor K 4096 48.1 -> 44.3,
 //    K 1024 33.6 -> 28.9, smoothed K 1024 22.7 -> 20.8, unicycle K 4096
-//    26.7 -> 24.6).  At least 5 samples: of a smaller tile the merge is the
-//    longer part; below 7, 256 threads (unicycle K 256 20.6 -> 16.6);
+//    26.7 -> 24.6).  Of tiles below 7 samples the merge is the longer part, so
+//    at least 5 on 256 threads (unicycle K 256 20.6 -> 16.6), unless a sample
+//    has kChainPoints points or more: then the chain is, and smaller tiles of
+//    512 threads win (quadrotor K 115, T 211, J 178 125.6 -> 70.7 us, K 195,
+//    T 104, J 186 87.4 -> 57.5; below the line K 142, T 37, J 0 18.6 against
+//    20.7.  Of 167 drawn problems with K up to 912 none is over 5 % slower
+//    than with two CTAs of 256 threads per SM, and they take 0.87 of it);
 //  - up to 64, two CTAs of 256 threads on each SM, up to 96 three, still one
 //    wave (vehicle K 9973, T 73 132 -> 103; the quadrotor at K 8192 takes 57.6
 //    with two and 56.6 with three, but 70 and 73 a call with host inputs,
 //    which every CTA reads over the host link);
 //  - beyond, several waves of 31 (unicycle K 65536 335 -> 286, quadrotor
 //    K 32768 707 -> 684).
-// From 12 on, S avoids multiples of 4: the scans read a sample's steps S
-// words of 8 or 16 bytes apart, and those strides fold the lanes onto a few
-// shared-memory banks (S 32 against 31 is the unicycle's 335 against 286).
+// From 12 on, S avoids multiples of 4 where a sample more keeps the wave: the
+// scans read a sample's steps S words of 8 or 16 bytes apart, and those strides
+// fold the lanes onto a few shared-memory banks (S 32 against 31 is the
+// unicycle's 335 against 286).  Of 32 one less would begin another wave (K 14562,
+// T 10, J 170: 43.6 us with 32, 58.1 with 31).
 constexpr int kServeStatic = 16 << 10;  // bytes the serving kernel holds beyond its tile, at most
-constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31;
-void default_shape(int K, int sms, int* S, int* threads) {
-  if (K <= 32 * sms) {
-    *S = std::max(kTileMin, (K + sms - 1) / sms);
-    *threads = *S >= kTileWide ? 512 : 256;
+constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31, kChainPoints = 400;
+void default_shape(int K, int points, int sms, int* S, int* threads) {
+  const int one = (K + sms - 1) / sms;
+  if (one < kTileWide && points < kChainPoints) {
+    *S = std::max(kTileMin, one);
+    *threads = 256;
+  } else if (one <= 32) {
+    *S = one;
+    *threads = 512;
   } else {
     const int per_sm = K <= 64 * sms ? 2 : 3;
     *S = K <= 96 * sms ? (K + per_sm * sms - 1) / (per_sm * sms) : kTileLarge;
     *threads = 256;
   }
-  if (*S >= 12 && *S % 4 == 0) *S += *S < 32 ? 1 : -1;
+  if (*S >= 12 && *S < 32 && *S % 4 == 0) ++*S;
   *S = std::min(*S, K);
 }
 
@@ -487,15 +498,19 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
   const bool fixed_S = t.samples_per_cta > 0;
   if (!fixed_S) {
     int threads = 0;
-    default_shape(p->K, sms, &t.samples_per_cta, &threads);
-    if (t.threads <= 0) t.threads = threads;
+    default_shape(p->K, p->T * p->n_shape, sms, &t.samples_per_cta, &threads);
     // a context takes its obstacles later: tiles larger than two per SM make
-    // leave room for the largest set
+    // leave room for the largest set.  Smaller ones on one CTA per SM would begin
+    // a second wave, so then it is two per SM (unicycle K 4000, T 256, J 200:
+    // 103 us with two of 14 samples, 131 with 182 CTAs of 22)
     const int two = std::min(32, (p->K + 2 * sms - 1) / (2 * sms));
-    while (t.samples_per_cta > two &&
-           smem_layout(p->T, t.samples_per_cta, p->n_shape, MPPI_MAX_OBSTACLES, n, 256,
-                       t.threads / 32, 0, batched).total > max_smem_optin())
-      --t.samples_per_cta;
+    if (t.samples_per_cta > two &&
+        smem_layout(p->T, t.samples_per_cta, p->n_shape, MPPI_MAX_OBSTACLES, n, 256,
+                    (t.threads > 0 ? t.threads : threads) / 32, 0, batched).total > max_smem_optin()) {
+      t.samples_per_cta = two;
+      threads = 256;
+    }
+    if (t.threads <= 0) t.threads = threads;
   }
   if (t.samples_per_cta > 32) return fail(MPPI_EINVAL, "samples_per_cta must be <= 32");
   if (t.threads <= 0) t.threads = 256;
