@@ -79,13 +79,13 @@ __global__ void draws_kernel(int K, int T, uint32_t k0, uint32_t k1, uint32_t it
 using StepFn = void (*)(CtrlDesc, const double*, const double*);
 
 StepFn pick_kernel(int model, int npos, bool r80, bool far) {
-  // [model][points 8 / 14][96 registers, 96 with far-field cells, 80 (with them)]
-  static const StepFn table[MPPI_NUM_MODELS][2][3] = {
-      {{step_u8, step_u8_far, step_u8_r80}, {step_u14, step_u14_far, step_u14_r80}},
-      {{step_q8, step_q8_far, step_q8_r80}, {step_q14, step_q14_far, step_q14_r80}},
-      {{step_a8, step_a8_far, step_a8_r80}, {step_a14, step_a14_far, step_a14_r80}},
-      {{step_p8, step_p8_far, step_p8_r80}, {step_p14, step_p14_far, step_p14_r80}}};
-  return table[model][npos == 14 ? 1 : 0][r80 ? 2 : far ? 1 : 0];
+  // [model][points 8 / 14][96 registers, 96 with far-field cells, 80, 80 with them]
+#define DBM_STEP_ROW(m, np) {step_##m##np, step_##m##np##_far, step_##m##np##_r80, step_##m##np##_r80_far}
+  static const StepFn table[MPPI_NUM_MODELS][2][4] = {
+      {DBM_STEP_ROW(u, 8), DBM_STEP_ROW(u, 14)}, {DBM_STEP_ROW(q, 8), DBM_STEP_ROW(q, 14)},
+      {DBM_STEP_ROW(a, 8), DBM_STEP_ROW(a, 14)}, {DBM_STEP_ROW(p, 8), DBM_STEP_ROW(p, 14)}};
+#undef DBM_STEP_ROW
+  return table[model][npos == 14 ? 1 : 0][(r80 ? 2 : 0) + (far ? 1 : 0)];
 }
 
 // Forms of the step kernels beyond the plain one (96-register form, separate
@@ -272,7 +272,7 @@ int max_smem_optin() {
 // beyond the plain one need a query only for the chunk, and only where the
 // grid could hold more than one tile per CTA.
 struct PickMemo {
-  int model, npos, threads, smem, nTiles, chunk;
+  int model, npos, threads, smem, nTiles, row, chunk;
   bool far;
   StepFn fn;
 };
@@ -302,9 +302,12 @@ int prepare_step_kernels(int dev, int form, int model, bool far) {
 }
 
 // both: the kernels of the other choice of `far` are prepared as well, so that
-// a later call with more or fewer obstacles finds them ready.
+// a later call with more or fewer obstacles finds them ready.  row: tiles of a
+// CTA, 0 = the library's choice.  Several in a row take the kernels with cells,
+// which alone have the loop over them: in the others it cost registers (the
+// vehicle's grid form spilled 56 bytes).
 int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, int form, bool far,
-                       StepFn* out, int* chunk, bool both = false) {
+                       StepFn* out, int* chunk, bool both = false, int row = 0) {
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxPickDevices) return fail(MPPI_EINVAL, "device %d out of range", dev);
@@ -312,34 +315,36 @@ int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, i
   if (const int rc = prepare_step_kernels(dev, form, model, far)) return rc;
   if (both)
     if (const int rc = prepare_step_kernels(dev, form, model, !far)) return rc;
-  if (form != kFormPlain && chunk_of(nTiles, num_sms()) == 1) {
+  if (form != kFormPlain && row <= 1 && (row == 1 || chunk_of(nTiles, num_sms()) == 1)) {
     *out = pick_form_kernel(form, model, npos, far);
     *chunk = 1;
     return MPPI_OK;
   }
   PickMemo& m = g_pick_memo[dev][form];
   if (m.fn && m.far == far && m.model == model && m.npos == npos && m.threads == threads &&
-      m.smem == smem && m.nTiles == nTiles) {
+      m.smem == smem && m.nTiles == nTiles && m.row == row) {
     *out = m.fn;
     *chunk = m.chunk;
     return MPPI_OK;
   }
-  StepFn fn = form == kFormPlain ? pick_kernel(model, npos, false, far)
-                                 : pick_form_kernel(form, model, npos, far);
+  bool r80 = false;
+  auto kernel = [&](bool f) {
+    return form == kFormPlain ? pick_kernel(model, npos, r80, f) : pick_form_kernel(form, model, npos, f);
+  };
   int occ = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel(far), threads, smem));
   if (form == kFormPlain) {
-    const StepFn lo = pick_kernel(model, npos, true, far);
     int occ_lo = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_lo, lo, threads, smem));
-    if (occ_lo > occ && (long)nTiles > (long)occ * num_sms()) {
-      fn = lo;
-      occ = occ_lo;
-    }
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_lo, pick_kernel(model, npos, true, far),
+                                                     threads, smem));
+    r80 = occ_lo > occ && (long)nTiles > (long)occ * num_sms();
+    if (r80) occ = occ_lo;
   }
-  *chunk = chunk_of(nTiles, (long)std::max(occ, 1) * num_sms());
-  m = PickMemo{model, npos, threads, smem, nTiles, *chunk, far, fn};
-  *out = fn;
+  *chunk = row ? row : chunk_of(nTiles, (long)std::max(occ, 1) * num_sms());
+  if (*chunk > 1)
+    if (const int rc = prepare_step_kernels(dev, form, model, true)) return rc;
+  *out = kernel(far || *chunk > 1);
+  m = PickMemo{model, npos, threads, smem, nTiles, row, *chunk, far, *out};
   return MPPI_OK;
 }
 
@@ -803,14 +808,14 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   StepFn fn = nullptr;
   int chunk = 1;
   rc = choose_step_kernel(c->p.model, t.positions_per_thread, t.threads, smem, c->D.nTiles,
-                          step_form(c), nc > 0, &fn, &chunk);
+                          step_form(c), nc > 0, &fn, &chunk, false, c->row);
   if (rc) return rc;
   c->tl = t;
   c->smem = smem;
   c->nc = nc;
   c->fn = fn;
   set_cells(c->D, J, nc);
-  c->D.chunk = c->row ? c->row : chunk;
+  c->D.chunk = chunk;
   c->D.obst = c->d_obst;
   return MPPI_OK;
 }
@@ -842,7 +847,7 @@ int mppi_set_grid(mppi_ctx* c, const float* sdf, int32_t nx, int32_t ny, double 
   int rc = choose_step_kernel(c->p.model, c->tl.positions_per_thread, c->tl.threads, c->smem,
                               c->D.nTiles,
                               off ? (c->p.sgf_window > 0 ? kFormSgf : kFormPlain) : kFormGrid,
-                              c->nc > 0, &fn, &chunk);
+                              c->nc > 0, &fn, &chunk, false, c->row);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->last));  // no step in flight reads the old map
   float* nb = nullptr;
@@ -876,7 +881,7 @@ int mppi_set_grid(mppi_ctx* c, const float* sdf, int32_t nx, int32_t ny, double 
   cudaFree(c->d_grid);
   c->d_grid = nb;
   c->fn = fn;
-  c->D.chunk = c->row ? c->row : chunk;
+  c->D.chunk = chunk;
   return MPPI_OK;
 }
 
@@ -892,7 +897,7 @@ int mppi_debug_set_form(mppi_ctx* c, int32_t cells, int32_t tiles_per_cta) {
   if (rc) return rc;
   StepFn fn = nullptr;
   rc = choose_step_kernel(c->p.model, t.positions_per_thread, t.threads, smem, c->D.nTiles,
-                          step_form(c), nc > 0, &fn, &chunk);
+                          step_form(c), nc > 0, &fn, &chunk, false, tiles_per_cta);
   if (rc) return rc;
   c->cells = cells != 0;
   c->row = tiles_per_cta;
@@ -900,7 +905,7 @@ int mppi_debug_set_form(mppi_ctx* c, int32_t cells, int32_t tiles_per_cta) {
   c->nc = nc;
   set_cells(c->D, c->D.J, nc);
   c->fn = fn;
-  c->D.chunk = c->row ? c->row : chunk;
+  c->D.chunk = chunk;
   return MPPI_OK;
 }
 
@@ -1085,7 +1090,9 @@ int mppi_get_tiling(mppi_ctx* c, mppi_tiling* t, int32_t* n_ctas) {
 int mppi_get_kernel_regs(mppi_ctx* c, int32_t* regs_cap) {
   if (!c) return fail(MPPI_ESTATE, "context is NULL");
   if (!regs_cap) return fail(MPPI_EINVAL, "regs_cap is NULL");
-  const bool r80 = c->fn == pick_kernel(c->p.model, c->tl.positions_per_thread, true, c->nc > 0);
+  bool r80 = false;
+  for (bool far : {false, true})
+    r80 = r80 || c->fn == pick_kernel(c->p.model, c->tl.positions_per_thread, true, far);
   *regs_cap = r80 ? DBM_STEP_MAXNREG_R80 : DBM_STEP_MAXNREG;
   return MPPI_OK;
 }

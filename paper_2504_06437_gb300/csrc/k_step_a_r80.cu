@@ -1,5 +1,5 @@
 // One-controller step kernels of the Ackermann vehicle (Eq. 14), 80-register form
-// (see DBM_STEP_MAXNREG_R80).
+// (see DBM_STEP_MAXNREG_R80), without and with far-field cells.
 #include "kernels.cuh"
 
 namespace dbm {
@@ -7,12 +7,24 @@ namespace dbm {
 __global__ void __maxnreg__(DBM_STEP_MAXNREG_R80) step_a8_r80(const __grid_constant__ CtrlDesc D,
                                                      const double* __restrict__ x0,
                                                      const double* __restrict__ xref) {
-  step_body<2, 8, false, false, true>(D, x0, xref);
+  step_body<2, 8>(D, x0, xref);
 }
 
 __global__ void __maxnreg__(DBM_STEP_MAXNREG_R80) step_a14_r80(const __grid_constant__ CtrlDesc D,
                                                       const double* __restrict__ x0,
                                                       const double* __restrict__ xref) {
+  step_body<2, 14>(D, x0, xref);
+}
+
+__global__ void __maxnreg__(DBM_STEP_MAXNREG_R80) step_a8_r80_far(
+    const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,
+    const double* __restrict__ xref) {
+  step_body<2, 8, false, false, true>(D, x0, xref);
+}
+
+__global__ void __maxnreg__(DBM_STEP_MAXNREG_R80) step_a14_r80_far(
+    const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,
+    const double* __restrict__ xref) {
   step_body<2, 14, false, false, true>(D, x0, xref);
 }
 

@@ -100,9 +100,15 @@ __global__ void step_p8_grid(const __grid_constant__ CtrlDesc D, const double* _
 __global__ void step_p14_grid(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,
                               const double* __restrict__ xref);
 
-// The 96-register forms with the far-field cells compiled in (suffix _far),
-// launched only for problems that use them.
+// The same with the far-field cells and several tiles in a row compiled in
+// (suffix _far), launched only for problems that use either.
 #define DBM_STEP_FAR(m)                                                                          \
+  __global__ void step_##m##8_r80_far(const __grid_constant__ CtrlDesc D,                         \
+                                      const double* __restrict__ x0,                              \
+                                      const double* __restrict__ xref);                           \
+  __global__ void step_##m##14_r80_far(const __grid_constant__ CtrlDesc D,                        \
+                                       const double* __restrict__ x0,                             \
+                                       const double* __restrict__ xref);                          \
   __global__ void step_##m##8_far(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0,  \
                                   const double* __restrict__ xref);                               \
   __global__ void step_##m##14_far(const __grid_constant__ CtrlDesc D, const double* __restrict__ x0, \

@@ -880,10 +880,11 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
 // The batch kernels carry it, and the one-controller kernels have a form
 // with it and one without, so that controllers that do not smooth run code
 // with no trace of it.
-// FAR: far-field cells are compiled in (taken when D.nc is set).  The
-// 96-register one-controller kernels have a form with them and one without:
-// a small step after an L2 flush fetches its code from memory, and with the
-// cells' code in the kernel, though not taken, it was 3 to 7 us longer.
+// FAR: far-field cells are compiled in (taken when D.nc is set), and in the
+// one-controller kernels the loop over several tiles.  Those have a form with
+// both and one without: a small step after an L2 flush fetches its code from
+// memory, and with the cells' code in the kernel, though not taken, it was 3 to
+// 7 us longer; the loop alone made the grid form spill (35.5 against 27.3 us).
 // The one-controller kernels inline the body (run_tile_inl), so the
 // descriptor stays the kernel's own parameter: its fields are read from the
 // parameter bank, and no store in the body can alias them.  The batch
@@ -918,7 +919,8 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   float* xi = reinterpret_cast<float*>(smem + L.xi);
   double* red = reinterpret_cast<double*>(smem + L.red);
   DevState* st = D.st;
-  const int t_end = min(tile0 + count, D.nTiles);  // this CTA's tiles: [tile0, t_end)
+  constexpr bool ROWS = BATCHED || FAR;  // several tiles in a row: compiled in with the cells
+  const int t_end = ROWS ? min(tile0 + count, D.nTiles) : tile0 + 1;  // this CTA's: [tile0, t_end)
 
   // ---- prologue: stage obstacles (TMA bulk copy), per-step constants
   __syncthreads();  // previous use of shared memory by this CTA is over
@@ -1066,7 +1068,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   }
   __syncthreads();
   // (one lane of the last warp, which has the fewest samples below)
-  if (tid == nthreads - 32 && tile == tile0) {
+  if (tid == nthreads - 32 && (!ROWS || tile == tile0)) {
     float fbd = 0.0f, fb0 = 0.0f;
     for (int w = 0; w < nwarps; ++w) {
       fbd += reinterpret_cast<const float*>(red)[2 * w];
@@ -1249,7 +1251,7 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   }
 
   __syncthreads();
-  if (++tile == t_end) break;
+  if (!ROWS || ++tile == t_end) break;
   }
 
   // ---- two-level last-arriver merge.  The CTA's writes are published by
