@@ -52,30 +52,33 @@ __device__ inline void sgf_weights(float* w, int W, int p, int tid, int nthreads
   }
 }
 
-// S_e = sum_{i<e} g^i = (1 - g^e) / (1 - g) and C_e = sum_{i=1..e} S_i for
-// 1 <= e <= MPPI_MAX_T, from the highest bit of e down: with p = g^m,
+// S_e = sum_{i<e} g^i = (1 - g^e) / (1 - g) for 1 <= e <= MPPI_MAX_T, and with
+// SUM C_e = sum_{i=1..e} S_i, from the highest bit of e down: with p = g^m,
 //   S_2m = S_m (1 + p),  C_2m = C_m (1 + p) + m S_m,
 //   S_(m+1) = 1 + g S_m, C_(m+1) = C_m + S_(m+1).
 // Every term is positive, so both are right to a few roundings however close
 // g is to 1, where the quotients cancel: at g = 1 - 1e-8 and e = 256 the form
 // (e - g S_e) / (1 - g) of C_e is 2e-5 off with pow and 1e-3 off with g^e by
-// repeated squaring.  Some twenty FP64 operations in a row.
-__device__ __forceinline__ double geometric_sums(double g, int e, double* C_out) {
-  double p = g, S = 1.0, C = 1.0;  // m = 1
-  int m = 1;
+// repeated squaring.  At most 32 FP64 operations for S_e, of which a warp's
+// take 16 cycles each; C_e is one thread's.
+template <bool SUM>
+__device__ __forceinline__ double geometric_sum(double g, int e, double* C_out) {
+  double p = g, S = 1.0, C = 1.0, m = 1.0;
   for (int bit = 31 - __clz(e); --bit >= 0;) {
-    C = C * (1.0 + p) + m * S;
-    S *= 1.0 + p;
+    if (SUM) C = fma(m, S, fma(C, p, C));
+    S = fma(S, p, S);
     p *= p;
-    m *= 2;
+    if (SUM) m += m;
     if ((e >> bit) & 1) {
-      S = 1.0 + g * S;
-      C += S;
+      S = fma(g, S, 1.0);
       p *= g;
-      ++m;
+      if (SUM) {
+        C += S;
+        m += 1.0;
+      }
     }
   }
-  *C_out = C;
+  if (SUM) *C_out = C;
   return S;
 }
 
@@ -85,13 +88,13 @@ __device__ __forceinline__ double geometric_sums(double g, int e, double* C_out)
 __device__ inline void init_constants(const CtrlDesc& D, int tid, int nthreads) {
   const int T = D.T;
   const double g = D.gamma_bas;
-  double C;
   for (int t = tid; t < T; t += nthreads) {
     // step t produces x_{t+1}: c_{t+1} = (1 - g^(T - t)) / (1 - g)
-    D.cw[t] = (float)(D.R_B_d * geometric_sums(g, T - t, &C));
+    D.cw[t] = (float)(D.R_B_d * geometric_sum<false>(g, T - t, nullptr));
   }
   if (tid == nthreads - 1) {
-    D.st->g1 = g * geometric_sums(g, T, &C);
+    double C;
+    D.st->g1 = g * geometric_sum<true>(g, T, &C);
     D.st->csum = C;
   }
   if (D.sgf_wp)
