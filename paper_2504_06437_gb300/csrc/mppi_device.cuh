@@ -74,7 +74,7 @@ struct DevState {
   double C0;         // sum_t gamma u_t^T (S_e Sigma)^-1 u_t of the next step
   double csum, g1;   // DBaS unrolling constants (see above)
   float L00, L10, L11;  // chol(S_e Sigma) of the next step
-  unsigned near;     // near obstacles of the tiles' cells (far_share); zero between steps
+  unsigned near;     // sum over the cells of their near obstacles' share, in 256ths; zero between steps
   unsigned long long iter;  // Philox counter words 2..3
   int first;         // 1 until the first step
   int status;        // kStatus*
@@ -611,10 +611,12 @@ __host__ __device__ constexpr int far_pos(int i, int k) {
 // the three-term recurrence of 1 / (1 - 2 x t + t^2); Q_n is homogeneous of
 // degree n, so its n + 1 coefficients follow from the two rows before.  Lanes
 // take obstacles; their sums are added across the warp with a transposing
-// butterfly (each lane ends with three of the coefficients).
+// butterfly (each lane ends with three of the coefficients).  The cell's share
+// of near obstacles goes to *near_share, if given (look_samples).
 template <bool BATCHED>
 __device__ __noinline__ void far_setup(int cell_off, int list_off, int pose_off, int obs_off, int u0,
-                                       int u1, int S, int J, float r_body, float h_eps, int lane) {
+                                       int u1, int S, int J, float r_body, float h_eps,
+                                       unsigned* near_share, int lane) {
   extern __shared__ __align__(16) char smem[];
   FarCell* cell = reinterpret_cast<FarCell*>(smem + cell_off);
   unsigned short* list = reinterpret_cast<unsigned short*>(smem + list_off);
@@ -672,6 +674,7 @@ __device__ __noinline__ void far_setup(int cell_off, int list_off, int pose_off,
     cell->cy = cy;
     cell->inv_R = inv_R;
     cell->n_near = direct ? -1 : nn;
+    if (near_share) atomicAdd(near_share, direct ? 256u : 256u * (unsigned)nn / (unsigned)J);
   }
   if (direct) return;
   float acc[48];

@@ -673,12 +673,15 @@ __device__ __forceinline__ void refine_list(const CtrlDesc& D, TileScratch& ts, 
   __syncthreads();
 }
 
-// A tile's share of near obstacles, in 256ths of its cells' obstacles, added to
-// the step's word.  Called by one warp, the cells set up.
+// The shares of near obstacles of a tile's cells, added to the step's sum by
+// one warp.  At 14 points per lane each cell's own warp adds its share instead
+// (far_setup), which leaves the tile's registers as they are: quadrotor K 32768,
+// J 500 672 -> 660 us; at 8 points it is this way 290 us against 293 (unicycle
+// K 65536, J 200).
 __device__ __forceinline__ void far_share(const CtrlDesc& D, const FarCell* cells, int nc, int lane) {
   const int nn = lane < nc ? cells[lane].n_near : 0;
   const unsigned near = __reduce_add_sync(0xffffffffu, (unsigned)(nn < 0 ? D.J : nn));
-  if (lane == 0) atomicAdd(&D.st->near, 256u * near / (unsigned)(nc * D.J));
+  if (lane == 0) atomicAdd(&D.st->near, 256u * near / (unsigned)D.J);
 }
 
 // How many samples the second look may take.  One CTA sums them alone, n of
@@ -692,13 +695,15 @@ __device__ __forceinline__ void far_share(const CtrlDesc& D, const FarCell* cell
 // the same bits; none where one sample has all the weight but 1 / kRefShare
 // or none can have that much; and none where the costs, and with them their
 // rounding, are small beside the temperature: at 4 lambda a rounding of the
-// cost moves a weight by 2^-22 of itself, as the exponential's own does.
-__device__ __forceinline__ int look_samples(const CtrlDesc& D, const TileScratch& ts,
-                                            unsigned share) {
-  if (!(ts.Z.hi > 1.0f + 1.0f / kRefShare) || ts.Z.hi > (float)kRefShare) return 0;
-  if (ts.ref * D.inv_lambda_f <= 4.0f) return 0;
-  const float near = (float)share / (256.0f * (float)D.nTiles);
-  return (int)fminf(D.look_max * (1.0f - near - D.look_over), (float)kRefMax);
+// cost moves a weight by 2^-22 of itself, as the exponential's own does.  (And
+// no more than the merge's scales, whose place their costs take.)
+__device__ __forceinline__ bool look_pays(const CtrlDesc& D, const TileScratch& ts) {
+  return ts.Z.hi > 1.0f + 1.0f / kRefShare && ts.Z.hi <= (float)kRefShare &&
+         ts.ref * D.inv_lambda_f > 4.0f;
+}
+__device__ __forceinline__ int look_samples(const CtrlDesc& D, unsigned share) {
+  const float near = (float)share / (256.0f * (float)D.nTiles * (float)D.nc);
+  return min((int)fminf(D.look_max * (1.0f - near - D.look_over), (float)kRefMax), max(D.nscl, 32));
 }
 
 // The clamped controls of the listed samples r0 .. r0 + Sc - 1, drawn anew
@@ -747,16 +752,16 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const int tid = threadIdx.x, nthreads = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
   const int T = D.T, P = D.P, J = D.J;
-  unsigned* word = &D.st->near;
-  const int n_max = look_samples(D, ts, __ldcg(word));
-  __syncthreads();
-  if (tid == 0) *word = 0u;  // for the next step
-  if (n_max <= 0) return;
+  if (!look_pays(D, ts)) {
+    if (tid == 0) D.st->near = 0u;  // for the next step
+    return;
+  }
+  const unsigned share = __ldcg(&D.st->near);  // its way is hidden behind the list's
   const SmemLayout L = smem_layout(T, D.S, P, J, Dyn<MODEL>::n, D.nscl, nwarps, D.nc, BATCHED);
   int* ref_k = reinterpret_cast<int*>(smem + L.red);
   float* delta = reinterpret_cast<float*>(smem + L.red) + kRefMax;
-  refine_list(D, ts, reinterpret_cast<const float*>(smem + L.scl), ref_k,
-              reinterpret_cast<int*>(smem + L.region), tid, nthreads);
+  float* above = reinterpret_cast<float*>(smem + L.scl);  // the scales; then cost less ts.ref
+  refine_list(D, ts, above, ref_k, reinterpret_cast<int*>(smem + L.region), tid, nthreads);
   const float2* Uf = reinterpret_cast<const float2*>(smem + L.Uf);
   const float* cw = reinterpret_cast<const float*>(smem + L.cw);
   float* scH = reinterpret_cast<float*>(smem + L.scH);
@@ -766,6 +771,8 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   float4* pose = reinterpret_cast<float4*>(smem + L.region);
   const float2* uB = reinterpret_cast<const float2*>(pose);
   const int n_ref = ts.n_ref;
+  const int n_max = look_samples(D, share);
+  if (tid == 0) D.st->near = 0u;
   if (n_ref == 0 || n_ref > n_max) return;
   for (int r0 = 0; r0 < n_ref; r0 += D.S) {
     const int Sc = min(D.S, n_ref - r0);
@@ -806,6 +813,7 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
         const FF c = ff_norm(ff_sum(FF{scH[s], scL[s]}, b));
         const double was = __ldcg(D.costs + ref_k[r0 + s]) - ts.base;
         delta[r0 + s] = (float)((double)c.hi + (double)c.lo - was);
+        above[r0 + s] = (float)(was - (double)ts.ref);
       }
     }
     __syncthreads();
@@ -819,8 +827,8 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
       const int i = lane + 32 * q;
-      was[q] = i < n_ref ? __ldcg(D.costs + ref_k[i]) - ts.base : 0.0;
-      e[q] = i < n_ref ? expf(-(float)(was[q] - (double)ts.ref) * D.inv_lambda_f) : 0.0f;
+      was[q] = i < n_ref ? __ldcg(D.costs + ref_k[i]) : 0.0;
+      e[q] = i < n_ref ? expf(-above[i] * D.inv_lambda_f) : 0.0f;
       se += e[q];
       if (i < n_ref) sd = fmaf(e[q], delta[i], sd);
     }
@@ -835,9 +843,9 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
     for (int q = 0; q < kPer; ++q) {
       const int i = lane + 32 * q;
       if (take && i < n_ref) {
-        const double now = was[q] + (double)(delta[i] - m);
-        D.costs[ref_k[i]] = ts.base + now;
-        delta[i] = expf(-(float)(now - (double)ts.ref) * D.inv_lambda_f) - e[q];
+        const float d = delta[i] - m;
+        D.costs[ref_k[i]] = was[q] + (double)d;
+        delta[i] = expf(-(above[i] + d) * D.inv_lambda_f) - e[q];
         ff_add(z, delta[i]);
       }
     }
@@ -1145,10 +1153,10 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
         const int g0 = (warp * NG + nc - 1) / nc, g1 = ((warp + 1) * NG + nc - 1) / nc;
         far_setup<BATCHED>(L.cell + warp * (int)sizeof(FarCell), L.list + 2 * warp * far_list_cap(J),
                            L.pose, L.obs4, g0 * gsz, min(g1 * gsz, T * S), S, J, D.r_body, D.h_eps,
-                           lane);
+                           NPOS == 14 ? &st->near : nullptr, lane);
       }
       __syncthreads();
-      if (warp == nwarps - 1) far_share(D, cells, nc, lane);
+      if (NPOS != 14 && warp == nwarps - 1) far_share(D, cells, nc, lane);
     }
   }
 
