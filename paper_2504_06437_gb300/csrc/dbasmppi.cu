@@ -536,7 +536,8 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
     // with far-field cells where they fit the persistent kernels' tile too,
     // whose rows are wider and whose serving form has 13 KB of its own: a
     // controller takes them alone, batched and served or not at all
-    int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads);
+    int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads,
+                       sms);
     if (!cells) nc = 0;
     if (nc > 0 && smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, nc,
                               true).total > limit - kServeStatic)
@@ -560,10 +561,12 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
 }
 
 // The obstacle count and the cells that go with it.
-void set_cells(CtrlDesc& D, int J, int nc) {
+void set_cells(CtrlDesc& D, int J, int nc, int threads) {
   D.J = J;
   D.nc = nc;
-  D.look_max = 0.5f * (float)D.K / (float)num_sms();
+  D.look_min = std::min(3, D.K / (2 * num_sms()));
+  // (a CTA of fewer than 256 threads sums the samples more slowly)
+  D.look_max = 0.9f * (float)D.K / (float)num_sms() * std::min(1.0f, (float)threads / 256.0f);
   D.look_over = nc > 0 ? (17.0f + far_setup_ops(nc, J, D.T * D.S * D.P)) / (float)J : 0.0f;
 }
 
@@ -814,7 +817,7 @@ int mppi_set_obstacles(mppi_ctx* c, const double* cxcyr, int32_t J) {
   c->smem = smem;
   c->nc = nc;
   c->fn = fn;
-  set_cells(c->D, J, nc);
+  set_cells(c->D, J, nc, t.threads);
   c->D.chunk = chunk;
   c->D.obst = c->d_obst;
   return MPPI_OK;
@@ -903,7 +906,7 @@ int mppi_debug_set_form(mppi_ctx* c, int32_t cells, int32_t tiles_per_cta) {
   c->row = tiles_per_cta;
   c->smem = smem;
   c->nc = nc;
-  set_cells(c->D, c->D.J, nc);
+  set_cells(c->D, c->D.J, nc, t.threads);
   c->fn = fn;
   c->D.chunk = chunk;
   return MPPI_OK;
@@ -1318,7 +1321,7 @@ extern "C" int mppi_step_static(const mppi_params* p, const double* d_obst, int3
   c.d_coll = (uint8_t*)(base + o_coll);
   c.d_Ustar = (double*)(base + o_Ustar);
   fill_desc(&c);
-  set_cells(c.D, J, c.nc);
+  set_cells(c.D, J, c.nc, c.tl.threads);
   c.D.chunk = chunk;
   c.D.ctl_out = d_ctl;
   c.D.u0_out = d_u0;
@@ -1706,7 +1709,7 @@ int batch_write_desc(mppi_batch* b, int slot) {
   c.nc = s.nc;
   slot_layout(b, s, &c);
   fill_desc(&c);
-  set_cells(c.D, s.J, s.nc);
+  set_cells(c.D, s.J, s.nc, s.tl.threads);
   s.D = c.D;
   CK(cudaMemcpy(b->d_descs + slot, &s.D, sizeof(CtrlDesc), cudaMemcpyHostToDevice));
   return MPPI_OK;

@@ -108,7 +108,8 @@ struct CtrlDesc {
   int chunk;                 // tiles of a CTA of the one-controller kernels
   int nc;                    // far-field cells of a tile (far_cells), 0 = every pair directly
   float r_body;              // largest distance of a shape point from the body's position
-  float look_max, look_over; // bounds of the second look (look_samples)
+  int look_min;              // bounds of the second look (look_samples)
+  float look_max, look_over;
   float dt, h_eps, C_coll, ln_mu, ln_sigma;
   float umin[2], umax[2];
   float Q[kMaxN], Qf[kMaxN];
@@ -223,14 +224,19 @@ __host__ __device__ inline int far_list_cap(int J) {
 // the whole step is about 8 us of the GPU, what the last CTA's second look
 // (refine_samples) takes when it is needed: the quadrotor at K 4096, T 50,
 // J 40 (2e7) took 71.5 us a call without cells, 72 to 80 us with them; at
-// K 8192, T 40, J 60 (7e7) 104 us without, 86 to 92 us with them.
+// K 8192, T 40, J 60 (7e7) 104 us without, 86 to 92 us with them.  None either
+// with fewer than kFarMinPerSm samples per SM: there two samples of the second
+// look take half as long as the whole step without cells, and cells save
+// little (0.72 to 0.99 of the time over 14 drawn problems).
 constexpr int kFarCellPoints = 1024;
+constexpr int kFarMinPerSm = 4;
 constexpr float kFarMinSaved = 4.0e7f;
 __host__ __device__ inline float far_setup_ops(int nc, int J, int pts) {
   return nc * (2800.0f + 53.0f * J) / pts;
 }
 __host__ __device__ inline int far_cells(int K, int T, int S, int P, int J, int npos,
-                                         int nthreads) {
+                                         int nthreads, int sms) {
+  if (K < kFarMinPerSm * sms) return 0;
   const int gsz = 32 * (npos / P);
   const int groups = (T * S + gsz - 1) / gsz;
   const int pts = T * S * P;

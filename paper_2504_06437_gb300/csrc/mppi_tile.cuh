@@ -684,26 +684,31 @@ __device__ __forceinline__ void far_share(const CtrlDesc& D, const FarCell* cell
   if (lane == 0) atomicAdd(&D.st->near, 256u * near / (unsigned)D.J);
 }
 
-// How many samples the second look may take.  One CTA sums them alone, n of
-// them in about n sms / K of the time that the direct evaluation of the whole
-// step takes, of which the cells saved the far obstacles' share less the
-// polynomials' and their set-up's (far_cells; look_over): at most half of what
-// was saved is given back.  Without a bound, at high temperatures, a vehicle at
-// K 221, T 132, J 378 took 654 us a step against 113 us without cells, one at
-// K 1076, T 156, J 577 913 us against 310 us.
-// None where every cell took its obstacles directly, where the direct sums are
-// the same bits; none where one sample has all the weight but 1 / kRefShare
-// or none can have that much; and none where the costs, and with them their
-// rounding, are small beside the temperature: at 4 lambda a rounding of the
-// cost moves a weight by 2^-22 of itself, as the exponential's own does.  (And
-// no more than the merge's scales, whose place their costs take.)
+// Whether the second look can matter: not where every weight but 1 / kRefShare
+// is one sample's or none can be as large as that, and not where the costs are
+// small beside the temperature.  The two sums of a cost differ by some 2^-26 of
+// it, so up to kLookCost lambda by some 2^-20 lambda, which is what they move
+// a weight by.  (Quadrotor K 15636, T 21, J 196, smallest cost 10 lambda: 98 us
+// with the look, 69 without.)
+// How many samples it may take: one CTA sums them alone, n of them in about
+// n sms / K of the time that the direct evaluation of the whole step takes, of
+// which the cells saved the far obstacles' share less the polynomials' and
+// their set-up's (far_cells; look_over).  At most nine tenths of what was saved
+// are given back, but up to three samples may take half of the direct time.
+// Without a bound, at high temperatures, a vehicle at K 1076, T 156, J 577 took
+// 913 us a step against 310 us without cells.  None where every cell took its
+// obstacles directly, where the direct sums are the same bits; and no more than
+// the merge's scales, whose place their costs take.
+constexpr float kLookCost = 64.0f;
 __device__ __forceinline__ bool look_pays(const CtrlDesc& D, const TileScratch& ts) {
   return ts.Z.hi > 1.0f + 1.0f / kRefShare && ts.Z.hi <= (float)kRefShare &&
-         ts.ref * D.inv_lambda_f > 4.0f;
+         ts.ref * D.inv_lambda_f > kLookCost;
 }
 __device__ __forceinline__ int look_samples(const CtrlDesc& D, unsigned share) {
   const float near = (float)share / (256.0f * (float)D.nTiles * (float)D.nc);
-  return min((int)fminf(D.look_max * (1.0f - near - D.look_over), (float)kRefMax), max(D.nscl, 32));
+  if (near >= 1.0f) return 0;
+  const float n = D.look_max * (1.0f - near - D.look_over);
+  return min(max((int)fminf(n, (float)kRefMax), D.look_min), max(D.nscl, 32));
 }
 
 // The clamped controls of the listed samples r0 .. r0 + Sc - 1, drawn anew
