@@ -475,6 +475,7 @@ void free_ctx(mppi_ctx* c) {
 // fold the lanes onto a few shared-memory banks (S 32 against 31 is the
 // unicycle's 335 against 286).  Of 32 one less would begin another wave (K 14562,
 // T 10, J 170: 43.6 us with 32, 58.1 with 31).
+constexpr int kFarAlone = 64;           // obstacles that pay for cells at one CTA per SM
 constexpr int kServeStatic = 16 << 10;  // bytes the serving kernel holds beyond its tile, at most
 constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31, kChainPoints = 400;
 void default_shape(int K, int points, int sms, int* S, int* threads) {
@@ -542,6 +543,19 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
     if (nc > 0 && smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, nc,
                               true).total > limit - kServeStatic)
       nc = 0;
+    // nor where they would leave one CTA on an SM that else holds two, unless
+    // there are many obstacles to save (quadrotor K 41425, T 133, J 36: 549 us
+    // without, 755 with them; unicycle K 16259, T 137, J 50 111 and 148; vehicle
+    // K 7972, T 150, J 87 247 and 165)
+    if (nc > 0 && J < kFarAlone && t.threads < 512) {
+      auto ctas = [&](int cells_) {
+        const int kRest = 1280;  // of a CTA's shared memory beside the dynamic part, about
+        return (limit + kRest) /
+               (smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl, t.threads / 32, cells_,
+                            false).total + kRest);
+      };
+      if (ctas(nc) < 2 && ctas(0) >= 2) nc = 0;
+    }
     *nc_out = nc;
     const SmemLayout L = smem_layout(p->T, t.samples_per_cta, p->n_shape, J, n, nscl,
                                      t.threads / 32, nc, batched);
