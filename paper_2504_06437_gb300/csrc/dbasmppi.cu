@@ -947,9 +947,9 @@ bool capturing(cudaStream_t s) {
 // that is being captured cannot wait for an event from outside the capture,
 // and the graph may be launched on any stream: there the host waits.
 // (cudaStreamPerThread is one handle for the streams of several threads.)
-int order_step(mppi_ctx* c, cudaStream_t s) {
+int order_step(mppi_ctx* c, cudaStream_t s, bool captured) {
   if (!c->order) return MPPI_OK;
-  if (capturing(s)) {
+  if (captured) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     CK(cudaThreadExchangeStreamCaptureMode(&mode));
     const cudaError_t e = cudaEventSynchronize(c->order);
@@ -961,9 +961,9 @@ int order_step(mppi_ctx* c, cudaStream_t s) {
   return MPPI_OK;
 }
 
-int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream, bool mirror) {
-  cudaStream_t s = stream ? (cudaStream_t)stream : c->own;
-  if (const int rc = order_step(c, s)) return rc;
+int launch_step(mppi_ctx* c, const double* x0, const double* xref, cudaStream_t s, bool mirror,
+                bool captured) {
+  if (const int rc = order_step(c, s, captured)) return rc;
   if (mirror) {
     c->D.seq = (int)++c->seq;
     c->fn<<<(c->D.nTiles + c->D.chunk - 1) / c->D.chunk, c->tl.threads, c->smem, s>>>(c->D, x0, xref);
@@ -984,7 +984,8 @@ int launch_step(mppi_ctx* c, const double* x0, const double* xref, void* stream,
 int mppi_step_device(mppi_ctx* c, const double* d_x0, const double* d_xref, void* stream) {
   if (!c) return fail(MPPI_ESTATE, "context is NULL");
   if (!d_x0 || !d_xref) return fail(MPPI_EINVAL, "device x0 / xref must not be NULL");
-  return launch_step(c, d_x0, d_xref, stream, false);
+  cudaStream_t s = stream ? (cudaStream_t)stream : c->own;
+  return launch_step(c, d_x0, d_xref, s, false, c->order && capturing(s));
 }
 
 int mppi_step(mppi_ctx* c, const double* x0, const double* xref, void* stream) {
@@ -1005,7 +1006,7 @@ int mppi_step(mppi_ctx* c, const double* x0, const double* xref, void* stream) {
   }
   // (a captured step has no number of its own: each replay would leave the same)
   const bool live = !capturing(s);
-  const int rc = launch_step(c, c->h_in_dev[b], c->h_in_dev[b] + n, s, live);
+  const int rc = launch_step(c, c->h_in_dev[b], c->h_in_dev[b] + n, s, live, !live);
   if (rc) return rc;
   CK(cudaEventRecord(c->in_ev[b], s));
   if (live) c->order = c->in_ev[b];
