@@ -59,8 +59,8 @@ __device__ inline void sgf_weights(float* w, int W, int p, int tid, int nthreads
 // Every term is positive, so both are right to a few roundings however close
 // g is to 1, where the quotients cancel: at g = 1 - 1e-8 and e = 256 the form
 // (e - g S_e) / (1 - g) of C_e is 2e-5 off with pow and 1e-3 off with g^e by
-// repeated squaring.  At most 32 FP64 operations for S_e, of which a warp's
-// take 16 cycles each; C_e is one thread's.
+// repeated squaring.  At most 32 FP64 operations for S_e; C_e, twice as long,
+// is one thread's.
 template <bool SUM>
 __device__ __forceinline__ double geometric_sum(double g, int e, double* C_out) {
   double p = g, S = 1.0, C = 1.0, m = 1.0;
@@ -896,11 +896,16 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
 // The batch kernels carry it, and the one-controller kernels have a form
 // with it and one without, so that controllers that do not smooth run code
 // with no trace of it.
-// FAR: far-field cells are compiled in (taken when D.nc is set), and in the
-// one-controller kernels the loop over several tiles.  Those have a form with
-// both and one without: a small step after an L2 flush fetches its code from
-// memory, and with the cells' code in the kernel, though not taken, it was 3 to
-// 7 us longer; the loop alone made the grid form spill (35.5 against 27.3 us).
+// FAR: far-field cells are compiled in (taken when D.nc is set), and with them
+// the loop over several tiles.  The one-controller kernels have a form with both
+// and one without: a small step after an L2 flush fetches its code from memory,
+// and with the cells' code in the kernel, though not taken, it was 3 to 7 us
+// longer.  The loop alone makes the grid form spill (K 1024 after a flush 33.2
+// us, 26.7 without it) and takes registers from the 14-point barrier (quadrotor
+// K 4096 54.8 and 51.0 us); at 8 points the code with the loop, of which one
+// round runs, is the faster one (after a flush vehicle K 7000 44.5 us without it
+// and 39.9 with it, quadrotor K 4096 45.4 and 43.7, 5-state quadrotor K 1024
+// 25.2 and 21.1; only unicycle K 256 19.6 and 21.2).
 // The one-controller kernels inline the body (run_tile_inl), so the
 // descriptor stays the kernel's own parameter: its fields are read from the
 // parameter bank, and no store in the body can alias them.  The batch
@@ -935,7 +940,9 @@ __device__ __forceinline__ void run_tile_inl(const CtrlDesc& D, int tile0, int c
   float* xi = reinterpret_cast<float*>(smem + L.xi);
   double* red = reinterpret_cast<double*>(smem + L.red);
   DevState* st = D.st;
-  constexpr bool ROWS = BATCHED || FAR;  // several tiles in a row: compiled in with the cells
+  // the loop over several tiles in a row: with the cells, and at 8 points
+  // (measured both ways, see above)
+  constexpr bool ROWS = BATCHED || FAR || (NPOS == 8 && !GRID);
   const int t_end = ROWS ? min(tile0 + count, D.nTiles) : tile0 + 1;  // this CTA's: [tile0, t_end)
 
   // ---- prologue: stage obstacles (TMA bulk copy), per-step constants
