@@ -535,8 +535,9 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
     const int nGroups = (nTiles + GT - 1) / GT;
     const int nscl = GT > nGroups ? GT : nGroups;
     // with far-field cells where they fit the persistent kernels' tile too,
-    // whose rows are wider and whose serving form has 13 KB of its own: a
-    // controller takes them alone, batched and served or not at all
+    // whose rows are wider and whose serving form has 13 KB of its own: with the
+    // same launch shape a controller takes them alone, batched and served or not
+    // at all (a context whose shape is left open has another shape than a batch)
     int nc = far_cells(p->K, p->T, t.samples_per_cta, p->n_shape, J, t.positions_per_thread, t.threads,
                        sms);
     if (!cells) nc = 0;
