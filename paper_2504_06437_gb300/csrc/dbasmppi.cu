@@ -304,8 +304,8 @@ int prepare_step_kernels(int dev, int form, int model, bool far) {
 // both: the kernels of the other choice of `far` are prepared as well, so that
 // a later call with more or fewer obstacles finds them ready.  row: tiles of a
 // CTA, 0 = the library's choice.  Several in a row take the kernels with cells,
-// which alone have the loop over them: in the others it cost registers (the
-// vehicle's grid form spilled 56 bytes).
+// which all have the loop over them; of the others only those where it costs
+// nothing (run_tile_inl).
 int choose_step_kernel(int model, int npos, int threads, int smem, int nTiles, int form, bool far,
                        StepFn* out, int* chunk, bool both = false, int row = 0) {
   int dev = 0;
@@ -390,7 +390,8 @@ struct mppi_ctx {
   cudaEvent_t in_ev[2] = {nullptr, nullptr};
   bool in_ev_pending[2] = {false, false};
   int in_next = 0;
-  cudaEvent_t order = nullptr;  // in_ev of the last step, when it came from mppi_step
+  cudaEvent_t last_ev = nullptr;  // in_ev of the last step, when it came from mppi_step
+  cudaEvent_t order = nullptr;    // the same, once mppi_get_control has returned that step's results
   DevState* h_st = nullptr; // pinned readback
   double* h_U = nullptr;    // pinned readback
   HostOut* h_out = nullptr;      // mapped mirror of u0, status and the sequence, written by the step
@@ -975,7 +976,7 @@ int launch_step(mppi_ctx* c, const double* x0, const double* xref, cudaStream_t 
   }
   CK(cudaGetLastError());
   c->last = s;
-  c->order = nullptr;
+  c->last_ev = c->order = nullptr;
   c->stepped = true;
   c->mirrored = c->mirror_U = mirror;
   return MPPI_OK;
@@ -1010,7 +1011,7 @@ int mppi_step(mppi_ctx* c, const double* x0, const double* xref, void* stream) {
   const int rc = launch_step(c, c->h_in_dev[b], c->h_in_dev[b] + n, s, live, !live);
   if (rc) return rc;
   CK(cudaEventRecord(c->in_ev[b], s));
-  if (live) c->order = c->in_ev[b];
+  if (live) c->last_ev = c->in_ev[b];
   c->in_ev_pending[b] = true;
   c->in_next = b ^ 1;
   return MPPI_OK;
@@ -1040,6 +1041,7 @@ int mppi_get_control(mppi_ctx* c, double* u0, double* U) {
           u0[1] = o->u0[1];
         }
         if (U) memcpy(U, c->h_out + 1, sizeof(double) * 2 * c->p.T);
+        c->order = c->last_ev;  // the step may not have ended yet
         return MPPI_OK;
       }
       if ((n & 1023u) == 0u && cudaStreamQuery(c->last) != cudaErrorNotReady) break;
