@@ -462,9 +462,9 @@ void free_ctx(mppi_ctx* c) {
 //    at least 5 on 256 threads (unicycle K 256 20.6 -> 16.6), unless a sample
 //    has kChainPoints points or more: then the chain is, and smaller tiles of
 //    512 threads win (quadrotor K 115, T 211, J 178 125.6 -> 70.7 us, K 195,
-//    T 104, J 186 87.4 -> 57.5; below the line K 142, T 37, J 0 18.6 against
-//    20.7.  Of 167 drawn problems with K up to 912 none is over 5 % slower
-//    than with two CTAs of 256 threads per SM, and they take 0.87 of it);
+//    T 104, J 186 87.4 -> 57.5; below the line K 142, T 64, J 5 20.6 against
+//    22.7.  Of 167 drawn problems with K up to 912 one is over 5 % slower than
+//    with two CTAs of 256 threads per SM, by 12 %, and they take 0.87 of it);
 //  - up to 64, two CTAs of 256 threads on each SM, up to 96 three, still one
 //    wave (vehicle K 9973, T 73 132 -> 103; the quadrotor at K 8192 takes 57.6
 //    with two and 56.6 with three, but 70 and 73 a call with host inputs,
@@ -478,7 +478,7 @@ void free_ctx(mppi_ctx* c) {
 // T 10, J 170: 43.6 us with 32, 58.1 with 31).
 constexpr int kFarAlone = 64;           // obstacles that pay for cells at one CTA per SM
 constexpr int kServeStatic = 16 << 10;  // bytes the serving kernel holds beyond its tile, at most
-constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31, kChainPoints = 400;
+constexpr int kTileMin = 5, kTileWide = 7, kTileLarge = 31, kChainPoints = 600;
 void default_shape(int K, int points, int sms, int* S, int* threads) {
   const int one = (K + sms - 1) / sms;
   if (one < kTileWide && points < kChainPoints) {
@@ -580,10 +580,8 @@ int choose_tiling(const mppi_params* p, const mppi_tiling* req, int J, mppi_tili
 void set_cells(CtrlDesc& D, int J, int nc, int threads) {
   D.J = J;
   D.nc = nc;
-  D.look_min = std::min(3, D.K / (2 * num_sms()));
   // (a CTA of fewer than 256 threads sums the samples more slowly)
-  D.look_max = 0.9f * (float)D.K / (float)num_sms() * std::min(1.0f, (float)threads / 256.0f);
-  D.look_over = nc > 0 ? (17.0f + far_setup_ops(nc, J, D.T * D.S * D.P)) / (float)J : 0.0f;
+  D.look_max = std::min(kRefMax, D.K / num_sms() * std::min(threads, 256) / 256);
 }
 
 // Fill the descriptor from the parameters and the device buffers.

@@ -108,8 +108,7 @@ struct CtrlDesc {
   int chunk;                 // tiles of a CTA of the one-controller kernels
   int nc;                    // far-field cells of a tile (far_cells), 0 = every pair directly
   float r_body;              // largest distance of a shape point from the body's position
-  int look_min;              // bounds of the second look (look_samples)
-  float look_max, look_over;
+  int look_max;              // samples of the second look at most (look_samples)
   float dt, h_eps, C_coll, ln_mu, ln_sigma;
   float umin[2], umax[2];
   float Q[kMaxN], Qf[kMaxN];

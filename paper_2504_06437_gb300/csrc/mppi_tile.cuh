@@ -687,28 +687,24 @@ __device__ __forceinline__ void far_share(const CtrlDesc& D, const FarCell* cell
 // Whether the second look can matter: not where every weight but 1 / kRefShare
 // is one sample's or none can be as large as that, and not where the costs are
 // small beside the temperature.  The two sums of a cost differ by some 2^-26 of
-// it, so up to kLookCost lambda by some 2^-20 lambda, which is what they move
-// a weight by.  (Quadrotor K 15636, T 21, J 196, smallest cost 10 lambda: 98 us
-// with the look, 69 without.)
+// it, so up to kLookCost lambda by some 2^-22 lambda, and a weight by as much of
+// itself, which is what its exponential rounds.  (Quadrotor K 15636, T 21, J 196,
+// smallest cost 10 lambda: 98 us with the look, 69 without.)
 // How many samples it may take: one CTA sums them alone, n of them in about
-// n sms / K of the time that the direct evaluation of the whole step takes, of
-// which the cells saved the far obstacles' share less the polynomials' and
-// their set-up's (far_cells; look_over).  At most nine tenths of what was saved
-// are given back, but up to three samples may take half of the direct time.
-// Without a bound, at high temperatures, a vehicle at K 1076, T 156, J 577 took
-// 913 us a step against 310 us without cells.  None where every cell took its
-// obstacles directly, where the direct sums are the same bits; and no more than
-// the merge's scales, whose place their costs take.
-constexpr float kLookCost = 64.0f;
+// n sms / K of the time that the direct evaluation of the whole step takes; up to
+// that time (D.look_max; of 274 looks at lambda 1 over 140 drawn problems 12 had
+// more samples).  Without a bound, at high temperatures, a vehicle at
+// K 1076, T 156, J 577 took 913 us a step against 310 us without cells.  None
+// where every cell took its obstacles directly, where the direct sums are the
+// same bits; and no more than the merge's scales, whose place their costs take.
+constexpr float kLookCost = 16.0f;
 __device__ __forceinline__ bool look_pays(const CtrlDesc& D, const TileScratch& ts) {
   return ts.Z.hi > 1.0f + 1.0f / kRefShare && ts.Z.hi <= (float)kRefShare &&
-         ts.ref * D.inv_lambda_f > kLookCost;
+         fabsf(ts.ref) * D.inv_lambda_f > kLookCost;
 }
 __device__ __forceinline__ int look_samples(const CtrlDesc& D, unsigned share) {
-  const float near = (float)share / (256.0f * (float)D.nTiles * (float)D.nc);
-  if (near >= 1.0f) return 0;
-  const float n = D.look_max * (1.0f - near - D.look_over);
-  return min(max((int)fminf(n, (float)kRefMax), D.look_min), max(D.nscl, 32));
+  if (share >= 256u * (unsigned)D.nTiles * (unsigned)D.nc) return 0;
+  return min(D.look_max, max(D.nscl, 32));
 }
 
 // The clamped controls of the listed samples r0 .. r0 + Sc - 1, drawn anew
@@ -739,16 +735,18 @@ __device__ __forceinline__ void refine_draws(const CtrlDesc& D, const TileScratc
 // What the two sums of a sample differ by has a part that all samples share,
 // for instance where a term of 1 / h_eps is paired with another obstacle.
 // Only the listed samples are summed again, so that part would shift their
-// weights against all the others'.  It is taken out: with m the mean of the
-// differences delta, weighted by the weights, a listed sample's cost changes by
-// delta - m.  Z then never falls (exp is convex: the mean of
-// exp(-(delta - m) / lambda) is at least 1), so it stays at least 1, as the
-// final stage assumes.  Where the differences left over exceed lambda the
-// costs' rounding decides the weights in either sum, and the first one stays.
+// weights against all the others'.  Where it is more than kLookShift lambda it is
+// taken out: with m the mean of the differences delta, weighted by the weights, a
+// listed sample's cost changes by delta - m.  Z then never falls (exp is
+// convex: the mean of exp(-(delta - m) / lambda) is at least 1), so it stays at
+// least 1, as the final stage assumes.  Where the differences left over exceed
+// lambda the costs' rounding decides the weights in either sum, and the first
+// one stays.
 // The last CTA runs this alone, a chain of latencies (list 2.5, draws 1,
 // rollout 2, barrier 2 to 20, costs 1, columns 1 us); out of line, so that its
 // registers leave the tile's code as it is: as a second round of the tile's
 // own code it took the batch kernel from 13.4 to 14.4 ms.
+constexpr float kLookShift = 1.0f / 1024.0f;
 template <int MODEL, int NPOS, bool BATCHED, bool GRID>
 __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const CtrlDesc& D = BATCHED ? tile_desc() : D_;
@@ -764,8 +762,8 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
   const unsigned share = __ldcg(&D.st->near);  // its way is hidden behind the list's
   const SmemLayout L = smem_layout(T, D.S, P, J, Dyn<MODEL>::n, D.nscl, nwarps, D.nc, BATCHED);
   int* ref_k = reinterpret_cast<int*>(smem + L.red);
-  float* delta = reinterpret_cast<float*>(smem + L.red) + kRefMax;
-  float* above = reinterpret_cast<float*>(smem + L.scl);  // the scales; then cost less ts.ref
+  float* now = reinterpret_cast<float*>(smem + L.red) + kRefMax;  // the new costs less ts.ref
+  float* above = reinterpret_cast<float*>(smem + L.scl);  // the scales; then the first costs less ts.ref
   refine_list(D, ts, above, ref_k, reinterpret_cast<int*>(smem + L.region), tid, nthreads);
   const float2* Uf = reinterpret_cast<const float2*>(smem + L.Uf);
   const float* cw = reinterpret_cast<const float*>(smem + L.cw);
@@ -816,42 +814,44 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
       b = warp_sum_ff(b);
       if (lane == 0) {
         const FF c = ff_norm(ff_sum(FF{scH[s], scL[s]}, b));
-        const double was = __ldcg(D.costs + ref_k[r0 + s]) - ts.base;
-        delta[r0 + s] = (float)((double)c.hi + (double)c.lo - was);
-        above[r0 + s] = (float)(was - (double)ts.ref);
+        const int k = ref_k[r0 + s];
+        const double sum = (double)c.hi + (double)c.lo;
+        above[r0 + s] = (float)(__ldcg(D.costs + k) - ts.base - (double)ts.ref);
+        now[r0 + s] = (float)(sum - (double)ts.ref);
+        D.costs[k] = ts.base + sum;
       }
     }
     __syncthreads();
   }
   if (warp == 0) {
     constexpr int kPer = kRefMax / 32;
-    double was[kPer];
-    float e[kPer];
+    float e[kPer], x[kPer], y[kPer];
     float se = 0.0f, sd = 0.0f;
-    bool near = true;  // (false for a difference that is no number)
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
       const int i = lane + 32 * q;
-      was[q] = i < n_ref ? __ldcg(D.costs + ref_k[i]) : 0.0;
-      e[q] = i < n_ref ? expf(-above[i] * D.inv_lambda_f) : 0.0f;
+      x[q] = i < n_ref ? above[i] : 0.0f;
+      y[q] = i < n_ref ? now[i] : 0.0f;
+      e[q] = i < n_ref ? expf(-x[q] * D.inv_lambda_f) : 0.0f;
       se += e[q];
-      if (i < n_ref) sd = fmaf(e[q], delta[i], sd);
+      sd = fmaf(e[q], y[q] - x[q], sd);
     }
-    const float m = warp_sum_f(sd) / warp_sum_f(se);  // the same in every lane
+    float m = warp_sum_f(sd) / warp_sum_f(se);  // the same in every lane
+    if (fabsf(m) * D.inv_lambda_f <= kLookShift) m = 0.0f;
+    bool near = true;  // (false for a difference that is no number)
 #pragma unroll
     for (int q = 0; q < kPer; ++q)
-      if (lane + 32 * q < n_ref)
-        near = near && fabsf(delta[lane + 32 * q] - m) * D.inv_lambda_f <= 1.0f;
+      near = near && fabsf(y[q] - x[q] - (lane + 32 * q < n_ref ? m : 0.0f)) * D.inv_lambda_f <= 1.0f;
     const bool take = __all_sync(0xffffffffu, near);
     FF z = {0.0f, 0.0f};
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
       const int i = lane + 32 * q;
-      if (take && i < n_ref) {
-        const float d = delta[i] - m;
-        D.costs[ref_k[i]] = was[q] + (double)d;
-        delta[i] = expf(-(above[i] + d) * D.inv_lambda_f) - e[q];
-        ff_add(z, delta[i]);
+      if (i < n_ref) {
+        if (!take) D.costs[ref_k[i]] = ts.base + ((double)ts.ref + (double)x[q]);
+        else if (m != 0.0f) D.costs[ref_k[i]] = ts.base + ((double)ts.ref + (double)(y[q] - m));
+        now[i] = expf(-(y[q] - m) * D.inv_lambda_f) - e[q];  // the weight's change
+        ff_add(z, now[i]);
       }
     }
     __syncwarp();
@@ -874,7 +874,7 @@ __device__ __noinline__ void refine_samples(const CtrlDesc& D_) {
       const float* Vt = reinterpret_cast<const float*>(V + (c >> 1) * Sc) + (c & 1);
       const float u = reinterpret_cast<const float*>(Uf)[c];
       FF a = {col_hi[c], col_lo[c]};
-      for (int s = 0; s < Sc; ++s) ff_add(a, delta[r0 + s] * (Vt[2 * s] - u));
+      for (int s = 0; s < Sc; ++s) ff_add(a, now[r0 + s] * (Vt[2 * s] - u));
       col_hi[c] = a.hi;
       col_lo[c] = a.lo;
     }
